@@ -400,6 +400,16 @@ int nrd_check_fastmath(const double* x, int64_t n, double* out, cudaStream_t str
  * Asynchronous.  Errors: NRD_EINVAL (null pointer, n < 0), NRD_ECUDA. */
 int nrd_check_narrow(const double* x, int64_t n, float* out, cudaStream_t stream);
 
+/* Check of the FP64 products the stencils form on the integer pipe (no
+ * counterpart in the paper): for n pairs of doubles x, y (device), out
+ * (device, 3n doubles) receives the integer-instruction product x y, CUDA's
+ * __dmul_rn of them, and the exponent-increment form of 2 x.  The first two
+ * are bit-identical where x, y and x y are each zero or normal, the third is
+ * exact where x is zero or normal and 2 x finite.
+ * Asynchronous.  Errors: NRD_EINVAL (null pointer, n < 0), NRD_ECUDA. */
+int nrd_check_softmul(const double* x, const double* y, int64_t n, double* out,
+                      cudaStream_t stream);
+
 /* Machine rates used as roofline denominators, measured on the current
  * device: FP64 and FP32 FMA throughput in TFLOP/s (an FMA counts 2 flops;
  * independent FMA chains on every SM) and device-to-device copy bandwidth in

@@ -42,6 +42,7 @@ def _compile(unit, verbose_ptxas=False):
 
 def build(force: bool = False, verbose_ptxas: bool = False) -> str:
     srcs = [os.path.join(SRC, u) for u in UNITS] + [os.path.join(SRC, "nrd_internal.h"),
+                                                  os.path.join(SRC, "softfp.h"),
                                                   os.path.join(HERE, "..", "include", "nrd.h")]
     if (not force and os.path.exists(OUT)
             and all(os.path.getmtime(OUT) >= os.path.getmtime(s) for s in srcs)):

@@ -113,9 +113,9 @@ int ctx_residual(nrd_ctx* c, const double* u, const double* b, double a0, double
   io.par = par;
   io.out = F;
   io.cfflux = c->d_cf;
-  io.pef = c->d_pef;   // the split form (every face once)
+  io.pef = c->d_pef;
   c->timer.begin(NRD_TK_RESIDUAL, s);
-  launch_stencil(H, c->mp, c->d_z, c->d_gz, ST_RESIDUAL, io, s, c->d_z3);
+  launch_stencil(H, c->mp, ST_RESIDUAL, io, s, c->d_z3);
   c->timer.end(NRD_TK_RESIDUAL, s);
   launch_reflux(H, io, ST_RESIDUAL, s);
   return check_launch(c);
@@ -140,8 +140,8 @@ int ctx_linearise(nrd_ctx* c, const double* u, const double* b, double a0, doubl
   io.par = par;
   pc_lin_targets(c->pc, &io.a32, &io.a64, &io.p2, &io.p2f);
   c->timer.begin(NRD_TK_LINEARISE, s);
-  io.pef = with_dz ? nullptr : c->d_pef;   // the split form (every face once)
-  launch_stencil(H, c->mp, c->d_z, c->d_gz, with_dz ? ST_LINZ : ST_LIN, io, s, c->d_z3);
+  io.pef = c->d_pef;
+  launch_stencil(H, c->mp, with_dz ? ST_LINZ : ST_LIN, io, s, c->d_z3);
   c->timer.end(NRD_TK_LINEARISE, s);
   launch_reflux(H, io, ST_RESIDUAL, s);
   c->timer.begin(NRD_TK_PC_SETUP, s);
@@ -195,12 +195,12 @@ int ctx_jv(nrd_ctx* c, const double* u, const double* v, const double* b, const 
     io.b = b;
     io.F0 = F0;
     io.eps = c->R.d_res + 0;
-    launch_stencil(H, c->mp, c->d_z, c->d_gz, ST_FD, io, s, c->d_z3);
+    launch_stencil(H, c->mp, ST_FD, io, s, c->d_z3);
     c->timer.end(NRD_TK_JV_FD, s);
     launch_reflux(H, io, ST_FD, s);
   } else {
     c->timer.begin(NRD_TK_JV, s);
-    launch_stencil(H, c->mp, c->d_z, c->d_gz, ST_JV, io, s, c->d_z3);
+    launch_stencil(H, c->mp, ST_JV, io, s, c->d_z3);
     c->timer.end(NRD_TK_JV, s);
     launch_reflux(H, io, ST_JV, s);
   }

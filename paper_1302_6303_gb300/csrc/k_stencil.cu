@@ -9,8 +9,10 @@
 //   k_avgdown      covered cells := mean of their children
 #include <algorithm>
 #include <cstdio>
+#include <type_traits>
 
 #include "nrd_internal.h"
+#include "softfp.h"
 
 namespace {
 
@@ -19,17 +21,14 @@ struct LevelH {
   double rh[NRD_MAX_LEVELS][3];   // 1/h
   double h3[NRD_MAX_LEVELS][3];   // 3h
   double kh[NRD_MAX_LEVELS][3];   // k/h
-  double kh5[NRD_MAX_LEVELS][3];  // 1.25 k/h
-  double bh2[NRD_MAX_LEVELS][3];  // beta/h^2 (linearisation only)
-  // the face fluxes' constants in terms of Ts = T_a + T_b (face_core)
-  double h12[NRD_MAX_LEVELS][3];  // 12h
-  double khs[NRD_MAX_LEVELS][3];  // 2^(-5/2) k/h
-  double kh5s[NRD_MAX_LEVELS][3]; // 2^(-3/2) 1.25 k/h
+  // constants of face_core
+  double c1[NRD_MAX_LEVELS][3];   // 1 / (12 h^2)
+  double cLh[NRD_MAX_LEVELS][3];  // (cL / 2) h
+  double cT[NRD_MAX_LEVELS][3];   // 2^(-5/2) k / h^2
 };
 
-// 2^(-5/2) and 2^(-3/2): Tf^(5/2) = 2^(-5/2) Ts^(5/2), Tf^(3/2) = 2^(-3/2) Ts^(3/2)
+// 2^(-5/2): Tf^(5/2) = 2^(-5/2) Ts^(5/2) with Ts = T_a + T_b
 constexpr double kP52 = 0.17677669529663688;
-constexpr double kP32 = 0.35355339059327376;
 
 struct GhostArgs {
   const uint8_t* gtype;
@@ -98,26 +97,23 @@ struct StArgs {
   const PatchDev* patches;
   const uint8_t* mask;
   const uint8_t* gtype;
-  const float* z;     // material z per cell
-  const float* gz;    // z of every ghost cell
-  const double* z3;   // z^3 of cells then ghosts (FP64), or null
+  const double* z3;   // z^3 of cells then ghosts (FP64)
+  bool soft;          // the faces' constants lie in the soft window
   int ntiles, N, G;
-  double k;       // D_T = k T^(5/2)
   double cL;      // limiter constant: 4 (Wilson form) or 2 (printed form)
-  double cL2;     // cL / 2 (face_core's Ts form)
-  double m15cL;   // -1.5 cL
   double R[6];
   LevelH lh;
   StencilIO io;
 };
 
-// Linearisation of one face at the iterate: the fluxes, the frozen
-// coefficients D_E = 2 Tf^3 S h / den and D_T = k Tf^(5/2) of Sec. 4.2, and
-// the partial derivatives of Phi_E w.r.t. E_a, E_b and T_a (= w.r.t. T_b) and
-// of Phi_T w.r.t. T_a, T_b (sign(0) = 0).
+// Linearisation of one face at the iterate, everything divided by h: the
+// fluxes, the P1 coefficients X = D_E / h^2 and T25 = D_T / h^2 of Sec. 4.2,
+// and the partial derivatives of Phi_E w.r.t. E_a, E_b and T_a (= w.r.t.
+// T_b), of Phi_T w.r.t. T_a, T_b, and of Phi_E w.r.t. z_a^3 (= z_b^3)
+// (sign(0) = 0).
 struct FaceLin {
   double PE, PT, aEa, aEb, aT, bTa, bTb, aZ;
-  double X, T25;   // C_E = X h, C_D = k 2^(-5/2) T25
+  double X, T25;
 };
 
 // 1/x from the PTX approximate FP64 reciprocal (rcp.approx.ftz.f64, a
@@ -157,11 +153,13 @@ __device__ __forceinline__ double rcp_nr(double x) {
 // e = 1 - x y0^2, 1/sqrt(x) = y0 (1 - e)^(-1/2) = y0 (1 + e/2 + 3 e^2/8 + ...),
 // a relative error of about (5/16) e^3 before rounding.  For x in the range
 // of rcp_nr; elsewhere the correctly rounded 1/sqrt(x).
+// SOFT (x in the soft window): the first product on the integer pipe.
+template <bool SOFT = false>
 __device__ __forceinline__ double rsqrt_nr(double x) {
   if (!in_refine_range(x)) return 1.0 / sqrt(x);
   const double y = rsqrt_approx(x);
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
+  const double e = fma(-Mul<SOFT>::pos(x, y), y, 1.0);
+  return fma(__dmul_rn(y, e), fma(0.375, e, 0.5), y);
 }
 
 // FP64 -> FP32 with round-to-nearest-even (the IEEE narrowing conversion,
@@ -187,7 +185,8 @@ __device__ __forceinline__ float narrow_rn(double x) {
   return __uint_as_float((hi & 0x80000000u) | (top - (896u << 23) + rnd));
 }
 
-// Face flux in the +e_d direction between cells a (low) and b (high):
+// Face flux in the +e_d direction between cells a (low) and b (high), over h
+// (its contribution to the divergence of a cell):
 //   Phi_E = D_E (E_b - E_a)/h with D_E = D_h/(1 + D_h g) (or the printed form)
 //         = 2 Tf^3 S dE / (3 h Zs S + cL Tf^3 |dE|),  S = E_a + E_b,
 //           Zs = z_a^3 + z_b^3, dE = E_b - E_a, Tf = (T_a + T_b)/2
@@ -195,71 +194,70 @@ __device__ __forceinline__ float narrow_rn(double x) {
 // with the intermediate quantities the partial derivatives reuse.  The
 // residual and the linearisation both take their fluxes from here, so the
 // two produce bit-identical residuals.
-// Evaluated in Ts = T_a + T_b = 2 Tf with the powers of 2 folded into the
-// constants (two FP64 multiplies fewer per face): with
-//   den' = 4 den = 12h Zs S + (cL/2) Ts^3 |dE|,   X = 2 Tf^3 S / den = Ts^3 S / den',
-//   Tf^(5/2) = 2^(-5/2) Ts^(5/2)  (2^(-5/2) in khs = 2^(-5/2) k/h).
-// rden = 1/den', hz = 12h Zs, ltadE = (cL/2) Ts^3 |dE| (4 times the Tf-form
-// terms), T15 = Ts^(3/2), T25 = Ts^(5/2), khT25 = (k/h) Tf^(5/2).
+// Evaluated in Ts = T_a + T_b = 2 Tf with the powers of 2 and h folded into
+// the constants c1 = 1/(12 h^2), cLh = (cL/2) h, cT = 2^(-5/2) k / h^2:
+//   Tc = c1 Ts^3, lt = Tc cLh |dE|, den = Zs S + lt, Q = Tc / den,
+//   Phi_E / h = X dE with X = Q S (= D_E / h^2),
+//   Phi_T / h = T25 dT with T25 = cT Ts^(5/2) (= D_T / h^2).
+// 13 FP64 instructions and 12 products; the products go to the integer pipe
+// where SOFT (the same bits, see softfp.h).  Both pipes then take about the
+// same time.  Measured at 256^3 (8x8x8 tiles): the linearisation's face launch
+// @LINF@, the residual's @RESF@.
 struct FaceCore {
-  double Ts, Ts2, Ts3, dE, adE, S, hz, ltadE, rden, X, PE, T15, T25, dT, khT25, PT;
+  double Ts, dE, S, r, Q, X, lt, PE, y, dT, T25, PT;
 };
+template <bool SOFT>
 __device__ __forceinline__ FaceCore face_core(double Ea, double Eb, double Ta, double Tb,
-                                              double za, double zb, double h12, double khs,
-                                              double cL2) {
+                                              double za, double zb, double c1, double cLh,
+                                              double cT) {
+  using M = Mul<SOFT>;
   FaceCore q;
-  q.Ts = Ta + Tb;
-  q.Ts2 = q.Ts * q.Ts;
-  q.Ts3 = q.Ts2 * q.Ts;
-  q.dE = Eb - Ea;
-  q.S = Ea + Eb;
-  q.hz = h12 * (za + zb);
-  q.adE = fabs(q.dE);
-  q.ltadE = (cL2 * q.Ts3) * q.adE;
-  q.rden = rcp_nr(fma(q.hz, q.S, q.ltadE));
-  q.X = (q.Ts3 * q.S) * q.rden;
-  q.PE = q.X * q.dE;
-  const double y = rsqrt_nr(q.Ts);
-  q.T15 = q.Ts2 * y;     // Ts^(3/2)
-  q.T25 = q.Ts * q.T15;  // Ts^(5/2)
-  q.dT = Tb - Ta;
-  q.khT25 = khs * q.T25;
-  q.PT = q.khT25 * q.dT;
+  q.Ts = __dadd_rn(Ta, Tb);
+  const double Ts3 = M::pos(M::pos(q.Ts, q.Ts), q.Ts);
+  q.dE = __dsub_rn(Eb, Ea);
+  q.S = __dadd_rn(Ea, Eb);
+  const double Tc = M::pos(c1, Ts3);
+  q.lt = M::any(Tc, M::any(cLh, fabs(q.dE)));
+  q.r = rcp_nr(fma(__dadd_rn(za, zb), q.S, q.lt));
+  q.Q = M::pos(Tc, q.r);
+  q.X = M::pos(q.Q, q.S);
+  q.PE = M::any(q.X, q.dE);
+  q.y = rsqrt_nr<SOFT>(q.Ts);
+  q.T25 = M::pos(cT, M::pos(Ts3, q.y));
+  q.dT = __dsub_rn(Tb, Ta);
+  q.PT = M::any(q.T25, q.dT);
   return q;
 }
 
 // Face flux of face_core and its partial derivatives at one iterate (the
-// frozen Jacobian), with X = 2 Tf^3 S / den, den = 3h Zs S + cL Tf^3 |dE|:
-//   PE = X dE (the P1 coefficient C_E = D_E h is X h)
-//   d PE / d E_a = (-4 Tf^3 E_a - PE (3h Zs - cL Tf^3 sg)) / den
-//   d PE / d E_b = ( 4 Tf^3 E_b - PE (3h Zs + cL Tf^3 sg)) / den
-//   d PE / d T_a = d PE / d T_b = Tf^2 (3 S dE - 1.5 cL |dE| PE) / den
-//   d PE / d Zs  = -PE 3h S / den
-//   PT = (k/h) Tf^(5/2) dT, d PT / d T_{a,b} = (k/h)(1.25 Tf^(3/2) dT -/+ Tf^(5/2))
-// (sg = sign(dE), sign(0) = 0), each evaluated in face_core's Ts form (the
-// factor 4 of den' cancels against the factor 4 of the Ts-form terms:
-// 4 Tf^3 = Ts^3 / 2, Tf^2 / den = Ts^2 / den').  The reciprocal and
-// Ts^(-1/2) come from rcp_nr / rsqrt_nr (within ~1e-13 relative of correctly
-// rounded arithmetic).  T25 is Ts^(5/2): C_D = k 2^(-5/2) T25.
+// frozen Jacobian).  With w = lt / den (so that Zs S / den = 1 - w):
+//   d PE / d E_a = Q (2 w E_b - S),  d PE / d E_b = Q (S - 2 w E_a)
+//   d PE / d T_a = d PE / d T_b = 3 (1 - w) PE / Ts
+//   d PE / d Zs  = -PE S / den
+//   d PT / d T_{a,b} = 2.5 PT / Ts -/+ T25
+// (from 4 Tf^3 S dE / den^2 and the like by dividing through by den; the terms
+// with sign(dE) combine with |dE|, so dE = 0 gives w = 0).  Ts^(-1) = y^2.
+template <bool SOFT>
 __device__ __forceinline__ FaceLin flux_lin(double Ea, double Eb, double Ta, double Tb, double za,
-                                            double zb, double h12, double khs, double kh5s,
-                                            double cL2, double m15cL, bool with_dz) {
-  const FaceCore q = face_core(Ea, Eb, Ta, Tb, za, zb, h12, khs, cL2);
+                                            double zb, double c1, double cLh, double cT,
+                                            bool with_dz) {
+  using M = Mul<SOFT>;
+  const FaceCore q = face_core<SOFT>(Ea, Eb, Ta, Tb, za, zb, c1, cLh, cT);
   FaceLin r;
   r.PE = q.PE;
-  r.X = q.X;
-  const double A = q.PE * q.hz;
-  const double Bs = q.X * q.ltadE;      // = 4 PE cL Tf^3 sign(dE)
-  const double t16 = q.Ts3 + q.Ts3;     // 16 Tf^3
-  r.aEa = (fma(-t16, Ea, Bs) - A) * q.rden;
-  r.aEb = (fma(t16, Eb, -Bs) - A) * q.rden;
-  r.aT = (q.Ts2 * q.rden) * fma(m15cL, q.adE * q.PE, 3.0 * (q.S * q.dE));
-  r.aZ = with_dz ? -(q.PE * q.rden) * (h12 * q.S) : 0.0;
-  r.T25 = q.T25;
   r.PT = q.PT;
-  const double khq = kh5s * q.T15 * q.dT;
-  r.bTa = khq - q.khT25;
-  r.bTb = khq + q.khT25;
+  r.X = q.X;
+  r.T25 = q.T25;
+  const double w = M::any(q.lt, q.r);
+  const double wQ2 = M::twice(M::any(w, q.Q));
+  r.aEa = fma(wQ2, Eb, -q.X);
+  r.aEb = fma(-wQ2, Ea, q.X);
+  const double rTs = M::pos(q.y, q.y);
+  r.aT = M::any(M::any(q.PE, rTs), fma(-3.0, w, 3.0));
+  const double PTr = M::any(q.PT, rTs);
+  r.bTa = fma(2.5, PTr, -q.T25);
+  r.bTb = fma(2.5, PTr, q.T25);
+  r.aZ = with_dz ? -(q.PE * q.r) * q.S : 0.0;
   return r;
 }
 
@@ -268,15 +266,20 @@ __device__ __forceinline__ FaceLin flux_lin(double Ea, double Eb, double Ta, dou
 //   c = sigma (T^4 - E), sigma = z^3 / T^3,
 // shared by the residual and the linearisation (bit-identical F); returns
 // 1/T and sigma for the partial derivatives.
+// (SOFT: E, T and z^3 in the soft window; the same bits either way.  At 256^3
+// the linearisation's cell launch 1.08 -> 0.72 ms, the residual's 0.89 ->
+// 0.63 ms.)
+template <bool SOFT>
 __device__ __forceinline__ void cell_balance(double a0, double dt, double E, double T, double z3,
                                              double bE, double bT, double divE, double divT,
                                              double& FE, double& FT, double& rT, double& sig) {
+  using M = Mul<SOFT>;
   rT = rcp_nr(T);
-  sig = z3 * rT * rT * rT;
-  const double T2 = T * T;
-  const double cp = sig * (T2 * T2 - E);
-  FE = a0 * E - bE - dt * (divE + cp);
-  FT = a0 * T - bT - dt * (divT - cp);
+  sig = M::pos(M::pos(M::pos(z3, rT), rT), rT);
+  const double T2 = M::pos(T, T);
+  const double cp = M::any(sig, fma(T2, T2, -E));
+  FE = fma(-dt, __dadd_rn(divE, cp), fma(a0, E, -bE));
+  FT = fma(-dt, __dsub_rn(divT, cp), fma(a0, T, -bT));
 }
 
 // Tangent of the face fluxes in the direction (dEa, dEb, dTa, dTb); sign(0) = 0.
@@ -335,20 +338,21 @@ __device__ __forceinline__ void put_scaled(const StencilIO& io, long NS, long sl
   }
 }
 
-// The linearisation's cell outputs (shared by the fused and the split form):
-// F from cell_balance, the coupling partials and the P2 data.
-template <bool DZ>
+// The linearisation's cell outputs: F from cell_balance, the coupling
+// partials and the P2 data.
+template <bool DZ, bool SOFT>
 __device__ __forceinline__ void lin_cell(const StencilIO& io, int N, int idx, double a0v,
                                          double dtv, double betav, float betaf, double E,
-                                         double T, double z, double divE, double divT) {
-  const double T2 = T * T, T3 = T2 * T;
+                                         double T, double z3, double divE, double divT) {
+  using M = Mul<SOFT>;
   double FE, FT, rT, sig;
-  cell_balance(a0v, dtv, E, T, z, io.b[idx], io.b[N + idx], divE, divT, FE, FT, rT, sig);
+  cell_balance<SOFT>(a0v, dtv, E, T, z3, io.b[idx], io.b[N + idx], divE, divT, FE, FT, rT, sig);
   io.out[idx] = FE;
   io.out[N + idx] = FT;
+  const double T2 = M::pos(T, T), T3 = M::pos(T2, T);
   // coupling tangent dc = cE vE + cT vT
   io.cc[idx] = -sig;
-  io.cc[N + idx] = sig * fma(3.0 * E, rT, T3);
+  io.cc[N + idx] = M::pos(sig, fma(M::pos(3.0, E), rT, T3));
   if (DZ) io.cc[2L * N + idx] = (T2 * T2 - E) * rT * rT * rT;   // d coupling / d z^3
   // P2 of Sec. 4.2 at this iterate: [[1 + sb, -sbt], [-sb, 1 + sbt]]
   // (det = (1 + sb)(1 + sbt) - sbt sb = 1 + sb + sbt), in the
@@ -399,12 +403,11 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
   constexpr int NFX = (TX + 1) * TY * TZ, NFY = TX * (TY + 1) * TZ, NFZ = TX * TY * (TZ + 1);
   constexpr int NC = TX * TY * TZ;
   constexpr bool TAN = (MODE == ST_JV);
-  constexpr bool LINF = (MODE == ST_LINF);     // the split linearisation's face launch
-  constexpr bool LINC = (MODE == ST_LINC);     // and its cell launch
-  constexpr bool FACES = LINF || MODE == ST_RESF;   // split forms: faces only
+  constexpr bool LIN = (MODE == ST_LINF || MODE == ST_LINZF);   // the linearisation's face launch
+  constexpr bool LINC = (MODE == ST_LINC || MODE == ST_LINZC);  // and its cell launch
+  constexpr bool FACES = LIN || MODE == ST_RESF;    // split forms: faces only
   constexpr bool CELLS = LINC || MODE == ST_RESC;   // split forms: cells only
-  constexpr bool LIN = (MODE == ST_LIN || MODE == ST_LINZ || LINF);   // writes the face data
-  constexpr bool DZ = (MODE == ST_LINZ);       // also the d/dz^3 partials
+  constexpr bool DZ = (MODE == ST_LINZF || MODE == ST_LINZC);   // also the d/dz^3 partials
   constexpr bool JVF = (MODE == ST_JVF);       // frozen-Jacobian Jv: sE, sT hold v
   extern __shared__ double smem[];
   double* sE = smem;
@@ -434,14 +437,6 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
     eps = *io.eps;
     reps = 1.0 / eps;
   }
-  // FP32 scale factors of the V-cycle coefficients per level and axis:
-  // beta C_E / h^2 = X (beta / h), beta C_T / h^2 = Ts^(5/2) (2^(-5/2) beta k / h^2)
-  __shared__ float s_bh[LIN ? NRD_MAX_LEVELS * 3 : 1], s_bk[LIN ? NRD_MAX_LEVELS * 3 : 1];
-  if (LIN && threadIdx.x < NRD_MAX_LEVELS * 3) {
-    const double rh = A.lh.rh[threadIdx.x / 3][threadIdx.x % 3];
-    s_bh[threadIdx.x] = (float)(betav * rh);
-    s_bk[threadIdx.x] = (float)(kP52 * (betav * A.k * rh * rh));
-  }
   const float betaf = (float)betav;
 
   for (int t = blockIdx.x; t < A.ntiles; t += gridDim.x) {
@@ -465,7 +460,6 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
       // the split forms' cell launch: the face fluxes come from pef (written
       // by the face launch, each face once), the divergence is formed in the
       // fused kernel's order, so F is bit-identical to it
-      const double rhx = A.lh.rh[lvl][0], rhy = A.lh.rh[lvl][1], rhz = A.lh.rh[lvl][2];
       const double* pE = io.pef;
       const double* pT = io.pef + NS;
       const int cex = CMP ? min(TX, nx - tile.i0) : TX, cey = CMP ? min(TY, ny - tile.j0) : TY;
@@ -478,7 +472,7 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
         const uint8_t m = A.mask[idx];
         if (m & MASK_COVERED) {
           if (LINC) {
-            lin_cell_covered<false>(io, N, idx);
+            lin_cell_covered<DZ>(io, N, idx);
           } else {
             io.out[idx] = 0.0;
             io.out[N + idx] = 0.0;
@@ -499,28 +493,33 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
         const long zl = (k == 0) ? gslot(4, i, j) : 2L * N + idx;
         const long zh = (k == nz - 1) ? gslot(5, i, j) : 2L * N + idx + (long)nx * ny;
         auto pick = [](bool skip, double v) { return skip ? 0.0 : v; };
-        const double divE = (pick(m & 4, pE[xh]) - pick(m & 2, pE[xl])) * rhx +
-                            (pick(m & 16, pE[yh]) - pick(m & 8, pE[yl])) * rhy +
-                            (pick(m & 64, pE[zh]) - pick(m & 32, pE[zl])) * rhz;
-        const double divT = (pick(m & 4, pT[xh]) - pick(m & 2, pT[xl])) * rhx +
-                            (pick(m & 16, pT[yh]) - pick(m & 8, pT[yl])) * rhy +
-                            (pick(m & 64, pT[zh]) - pick(m & 32, pT[zl])) * rhz;
+        const double divE = (pick(m & 4, pE[xh]) - pick(m & 2, pE[xl])) +
+                            (pick(m & 16, pE[yh]) - pick(m & 8, pE[yl])) +
+                            (pick(m & 64, pE[zh]) - pick(m & 32, pE[zl]));
+        const double divT = (pick(m & 4, pT[xh]) - pick(m & 2, pT[xl])) +
+                            (pick(m & 16, pT[yh]) - pick(m & 8, pT[yl])) +
+                            (pick(m & 64, pT[zh]) - pick(m & 32, pT[zl]));
         const double E = io.u[idx], T = io.u[N + idx];
-        const double z = A.z3 ? A.z3[idx] : (double)A.z[idx];
-        const double z3c = A.z3 ? z : z * z * z;
-        if (LINC) {
-          lin_cell<false>(io, N, idx, a0v, dtv, betav, betaf, E, T, z3c, divE, divT);
-        } else {
-          double FE, FT, rT, sig;
-          cell_balance(a0v, dtv, E, T, z3c, io.b[idx], io.b[N + idx], divE, divT, FE, FT, rT,
-                       sig);
-          io.out[idx] = FE;
-          io.out[N + idx] = FT;
-        }
+        const double z3c = A.z3[idx];
+        auto cell = [&](auto soft) {
+          constexpr bool SOFT = decltype(soft)::value;
+          if (LINC) {
+            lin_cell<DZ, SOFT>(io, N, idx, a0v, dtv, betav, betaf, E, T, z3c, divE, divT);
+          } else {
+            double FE, FT, rT, sig;
+            cell_balance<SOFT>(a0v, dtv, E, T, z3c, io.b[idx], io.b[N + idx], divE, divT, FE, FT,
+                               rT, sig);
+            io.out[idx] = FE;
+            io.out[N + idx] = FT;
+          }
+        };
+        if (soft_window(E) && soft_window(T) && soft_window(z3c)) cell(std::true_type{});
+        else cell(std::false_type{});
       }
       continue;
     }
     // ---- halo load (face halos only; edges and corners are never read)
+    bool soft_ok = A.soft;   // every staged value in the soft window
     for (int hh = threadIdx.x; hh < NH; hh += blockDim.x) {
       int hx_ = hh % HX, hy_ = (hh / HX) % HY, hz_ = hh / (HX * HY);
       int i = tile.i0 + hx_ - 1, j = tile.j0 + hy_ - 1, k = tile.k0 + hz_ - 1;
@@ -551,7 +550,7 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
         int idx = P.off + i + nx * (j + ny * k);
         e = io.u[idx];
         tt = io.u[N + idx];
-        z = A.z3 ? A.z3[idx] : (double)A.z[idx];
+        z = A.z3[idx];
         if (MODE == ST_JV || MODE == ST_FD) {
           ve = io.v[idx];
           vt = io.v[N + idx];
@@ -566,7 +565,7 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
         int gi = P.goff + P.fo[f] + a + nt1 * b;
         e = io.gu[gi];
         tt = io.gu[G + gi];
-        z = A.z3 ? A.z3[(long)N + gi] : (double)A.gz[gi];
+        z = A.z3[(long)N + gi];
         if (MODE == ST_JV || MODE == ST_FD) {
           ve = io.gv[gi];
           vt = io.gv[G + gi];
@@ -578,13 +577,16 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
       }
       sE[hh] = e;
       sT[hh] = tt;
-      sZ[hh] = A.z3 ? z : z * z * z;
+      sZ[hh] = z;
+      if (FACES) soft_ok = soft_ok && soft_window(e) && soft_window(tt) && soft_window(z);
       if (TAN) {
         svE[hh] = ve;
         svT[hh] = vt;
       }
     }
-    __syncthreads();
+    bool soft = false;   // block-uniform: the tile's products on the integer pipe
+    if (FACES) soft = __syncthreads_and(soft_ok);
+    else __syncthreads();
     // ---- face fluxes, each computed once per tile (split forms: once in the launch:
     // the low faces of the tile's cells, and the patch's high boundary faces
     // where the tile ends the patch, enumerated without gaps so that whole
@@ -603,6 +605,8 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
     const int nfxe = (ex + 1) * ey * tzl, nfye = ex * (ey + 1) * tzl;
     const int nfaces = FACES ? 3 * nlow + nbx + nby + nbz
                              : (CMP ? nfxe + nfye + ex * ey * (tzl + 1) : NFX + NFY + NFZ);
+    auto faces = [&](auto softc) {
+    constexpr bool SOFT = decltype(softc)::value;
     for (int f = threadIdx.x; f < nfaces; f += blockDim.x) {
       int dir, fi, fj, fk, slot = 0;
       double* outE = nullptr;
@@ -665,7 +669,7 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
       int hb = (fi + 1) + HX * ((fj + 1) + HY * (fk + 1));   // high-side cell
       int st = (dir == 0) ? 1 : ((dir == 1) ? HX : HX * HY);
       int ha = hb - st;                                      // low-side cell
-      const double h = A.lh.h[lvl][dir], h3 = A.lh.h3[lvl][dir], kh = A.lh.kh[lvl][dir];
+      const double h = A.lh.h[lvl][dir];
       double PE = 0.0, PT = 0.0;
       uint8_t gt = GT_SIBLING;
       int gi = -1;
@@ -707,24 +711,25 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
         int s = (pos == 0) ? -1 : 1;
         int hc = (pos == 0) ? hb : ha;      // the interior cell
         int ff = 2 * dir + (pos == nd ? 1 : 0);
+        const double rh = A.lh.rh[lvl][dir];
         if (TAN) {
-          PE = robin_tan(sE[hc], sT[hc], sZ[hc], h, A.R[ff], s, svE[hc], svT[hc]);
+          PE = rh * robin_tan(sE[hc], sT[hc], sZ[hc], h, A.R[ff], s, svE[hc], svT[hc]);
         } else {
-          PE = robin_flux(sE[hc], sT[hc], sZ[hc], h, A.R[ff], s);
+          PE = rh * robin_flux(sE[hc], sT[hc], sZ[hc], h, A.R[ff], s);
         }
         if (LIN) {
-          // dPhi/dE_c and dPhi/dT_c in slots 0 and 1; raw P1 slot holds D_b
+          // dPhi/dE_c and dPhi/dT_c over h in slots 0 and 1; raw P1 slot holds D_b
           double Ec = sE[hc], Tc = sT[hc], zc = sZ[hc];
           double Db = Tc * Tc * Tc / (3.0 * zc);
           double qd = 4.0 * Db + h;
           double rq = 1.0 / qd;
           double m = 2.0 * Ec - 8.0 * A.R[ff];
-          io.jc[fslot] = -(double)s * 2.0 * Db * rq;
-          io.jc[NS + fslot] = -(double)s * (Tc * Tc / zc) * m * h * rq * rq;
+          io.jc[fslot] = rh * (-(double)s * 2.0 * Db * rq);
+          io.jc[NS + fslot] = -(double)s * (Tc * Tc / zc) * m * rq * rq;
           io.jc[2 * NS + fslot] = 0.0;
           io.jc[3 * NS + fslot] = 0.0;
           io.jc[4 * NS + fslot] = 0.0;
-          if (DZ) io.jc[5 * NS + fslot] = (double)s * m * h * rq * rq * Db / zc;  // d Phi / d z_c^3
+          if (DZ) io.jc[5 * NS + fslot] = (double)s * m * rq * rq * Db / zc;  // d Phi / d z_c^3
           io.craw[fslot] = Db;
           io.craw[NS + fslot] = 0.0;
           put_scaled(io, NS, fslot, betav * 2.0 * Db * rq / h, 0.0);
@@ -732,12 +737,14 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
         PT = 0.0;
       } else {
         if (TAN) {
-          flux_tan(sE[ha], sE[hb], sT[ha], sT[hb], sZ[ha], sZ[hb], h3, kh, A.cL, svE[ha], svE[hb],
-                   svT[ha], svT[hb], PE, PT);
+          flux_tan(sE[ha], sE[hb], sT[ha], sT[hb], sZ[ha], sZ[hb], A.lh.h3[lvl][dir],
+                   A.lh.kh[lvl][dir], A.cL, svE[ha], svE[hb], svT[ha], svT[hb], PE, PT);
+          PE *= A.lh.rh[lvl][dir];
+          PT *= A.lh.rh[lvl][dir];
         } else if (LIN) {
-          FaceLin L = flux_lin(sE[ha], sE[hb], sT[ha], sT[hb], sZ[ha], sZ[hb],
-                               A.lh.h12[lvl][dir], A.lh.khs[lvl][dir], A.lh.kh5s[lvl][dir], A.cL2,
-                               A.m15cL, DZ);
+          FaceLin L = flux_lin<SOFT>(sE[ha], sE[hb], sT[ha], sT[hb], sZ[ha], sZ[hb],
+                                     A.lh.c1[lvl][dir], A.lh.cLh[lvl][dir], A.lh.cT[lvl][dir],
+                                     DZ);
           PE = L.PE;
           PT = L.PT;
           io.jc[fslot] = L.aEa;
@@ -746,20 +753,19 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
           io.jc[3 * NS + fslot] = L.bTa;
           io.jc[4 * NS + fslot] = L.bTb;
           if (DZ) io.jc[5 * NS + fslot] = L.aZ;
-          // only the scaled P1 coefficients: the coarsening averages them
-          // (raw values are kept for Robin faces alone)
+          // only the scaled P1 coefficients beta D / h^2: the coarsening
+          // averages them (raw values are kept for Robin faces alone)
           if (io.a32) {
-            io.a32[fslot] = narrow_rn(L.X) * s_bh[3 * lvl + dir];
-            io.a32[NS + fslot] = narrow_rn(L.T25) * s_bk[3 * lvl + dir];
+            io.a32[fslot] = narrow_rn(L.X) * betaf;
+            io.a32[NS + fslot] = narrow_rn(L.T25) * betaf;
           } else {
-            // beta D_E / h^2 = X beta / h, beta D_T / h^2 = Ts^(5/2) 2^(-5/2) beta k / h^2
-            const double bh = betav * A.lh.rh[lvl][dir];
-            io.a64[fslot] = L.X * bh;
-            io.a64[NS + fslot] = L.T25 * (kP52 * (bh * A.k * A.lh.rh[lvl][dir]));
+            io.a64[fslot] = L.X * betav;
+            io.a64[NS + fslot] = L.T25 * betav;
           }
         } else {
-          const FaceCore q = face_core(sE[ha], sE[hb], sT[ha], sT[hb], sZ[ha], sZ[hb],
-                                       A.lh.h12[lvl][dir], A.lh.khs[lvl][dir], A.cL2);
+          const FaceCore q = face_core<SOFT>(sE[ha], sE[hb], sT[ha], sT[hb], sZ[ha], sZ[hb],
+                                             A.lh.c1[lvl][dir], A.lh.cLh[lvl][dir],
+                                             A.lh.cT[lvl][dir]);
           PE = q.PE;
           PT = q.PT;
         }
@@ -776,10 +782,12 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
         outT[slot] = PT;
       }
     }
+    };
+    if (FACES && soft) faces(std::integral_constant<bool, FACES>{});
+    else faces(std::false_type{});
     __syncthreads();
     if (FACES) continue;   // the cell launch forms the balance
     // ---- cell balance
-    const double rhx = A.lh.rh[lvl][0], rhy = A.lh.rh[lvl][1], rhz = A.lh.rh[lvl][2];
     const int fex = CMP ? ex : TX, fey = CMP ? ey : TY;
     const int nce = CMP ? ex * ey * tzl : NC;
     for (int c = threadIdx.x; c < nce; c += blockDim.x) {
@@ -789,12 +797,8 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
       int idx = P.off + i + nx * (j + ny * k);
       uint8_t m = A.mask[idx];
       if (m & MASK_COVERED) {
-        if (LIN) {
-          lin_cell_covered<DZ>(io, N, idx);
-        } else {
-          io.out[idx] = 0.0;
-          io.out[N + idx] = 0.0;
-        }
+        io.out[idx] = 0.0;
+        io.out[N + idx] = 0.0;
         continue;
       }
       int xl = ci + (TX + 1) * (cj + TY * ck);
@@ -802,12 +806,12 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
       int zl = ci + TX * (cj + TY * ck);
       // coarse-side coarse-fine faces take their flux from flux matching
       auto pick = [](bool skip, double v) { return skip ? 0.0 : v; };
-      double divE = (pick(m & 4, fxE[xl + 1]) - pick(m & 2, fxE[xl])) * rhx +
-                    (pick(m & 16, fyE[yl + TX]) - pick(m & 8, fyE[yl])) * rhy +
-                    (pick(m & 64, fzE[zl + TX * TY]) - pick(m & 32, fzE[zl])) * rhz;
-      double divT = (pick(m & 4, fxT[xl + 1]) - pick(m & 2, fxT[xl])) * rhx +
-                    (pick(m & 16, fyT[yl + TX]) - pick(m & 8, fyT[yl])) * rhy +
-                    (pick(m & 64, fzT[zl + TX * TY]) - pick(m & 32, fzT[zl])) * rhz;
+      double divE = (pick(m & 4, fxE[xl + 1]) - pick(m & 2, fxE[xl])) +
+                    (pick(m & 16, fyE[yl + TX]) - pick(m & 8, fyE[yl])) +
+                    (pick(m & 64, fzE[zl + TX * TY]) - pick(m & 32, fzE[zl]));
+      double divT = (pick(m & 4, fxT[xl + 1]) - pick(m & 2, fxT[xl])) +
+                    (pick(m & 16, fyT[yl + TX]) - pick(m & 8, fyT[yl])) +
+                    (pick(m & 64, fzT[zl + TX * TY]) - pick(m & 32, fzT[zl]));
       int hc = (ci + 1) + HX * ((cj + 1) + HY * (ck + 1));
       double E = sE[hc], T = sT[hc], z = sZ[hc];
       double T2 = T * T, T3 = T2 * T;
@@ -822,15 +826,11 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
         double dc = sig * ((T3 + 3.0 * E * rT) * vT - vE);
         io.out[idx] = a0v * vE - dtv * (divE + dc);
         io.out[N + idx] = a0v * vT - dtv * (divT - dc);
-      } else if (LIN) {
-        lin_cell<DZ>(io, N, idx, a0v, dtv, betav, betaf, E, T, z, divE, divT);
       } else {
         double FE, FT, rT, sig;
-        cell_balance(a0v, dtv, E, T, z, io.b[idx], io.b[N + idx], divE, divT, FE, FT, rT, sig);
-        if (MODE == ST_FD) {
-          FE = (FE - io.F0[idx]) * reps;
-          FT = (FT - io.F0[N + idx]) * reps;
-        }
+        cell_balance<false>(a0v, dtv, E, T, z, io.b[idx], io.b[N + idx], divE, divT, FE, FT, rT, sig);
+        FE = (FE - io.F0[idx]) * reps;
+        FT = (FT - io.F0[N + idx]) * reps;
         io.out[idx] = FE;
         io.out[N + idx] = FT;
       }
@@ -844,34 +844,26 @@ struct RfArgs {
   const int* off;
   const int* face;
   const int4* g;
-  const PatchDev* patches;
   int nrf, N, G;
-  LevelH lh;
 };
 
 // Flux matching (Sec. 3.2.1): the coarse face flux is the average of the four
-// fine fluxes stored by the fine-side stencil; scale = -dt (RESIDUAL, JV) or
-// -dt/eps (FD).
-__global__ void k_reflux(RfArgs a, const int* __restrict__ rf_level, const double* cf,
-                         double* out, double dt, const double* par, const double* eps,
-                         int mode) {
+// fine fluxes stored by the fine-side stencil (each over the fine h, half the
+// coarse one: the coarse flux over its h is 1/8 of their sum); scale = -dt
+// (RESIDUAL, JV) or -dt/eps (FD).
+__global__ void k_reflux(RfArgs a, const double* cf, double* out, double dt, const double* par,
+                         const double* eps, int mode) {
   if (par) dt = par[1];
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < a.nrf; r += gridDim.x * blockDim.x) {
     int c = a.cell[r];
-    int lvl = rf_level[r];
     double sc = -dt;
     if (mode == ST_FD) sc /= *eps;
     double dE = 0.0, dT = 0.0;
     for (int q = a.off[r]; q < a.off[r + 1]; q++) {
-      int f = a.face[q];
-      int d = f / 2;
-      double s = (f % 2) ? 1.0 : -1.0;
+      double s = (a.face[q] % 2) ? 0.125 : -0.125;
       int4 g = a.g[q];
-      double PE = 0.25 * (cf[g.x] + cf[g.y] + cf[g.z] + cf[g.w]);
-      double PT = 0.25 * (cf[a.G + g.x] + cf[a.G + g.y] + cf[a.G + g.z] + cf[a.G + g.w]);
-      const double rh = a.lh.rh[lvl][d];   // 1/h: no FP64 division per face
-      dE += s * PE * rh;
-      dT += s * PT * rh;
+      dE += s * (cf[g.x] + cf[g.y] + cf[g.z] + cf[g.w]);
+      dT += s * (cf[a.G + g.x] + cf[a.G + g.y] + cf[a.G + g.z] + cf[a.G + g.w]);
     }
     out[c] += sc * dE;
     out[a.N + c] += sc * dT;
@@ -1028,7 +1020,16 @@ __global__ void k_check_narrow(const double* x, long n, float* out) {
   }
 }
 
-LevelH level_h(const Hier& H, double k = 0.01, double beta = 0.0) {
+__global__ void k_check_softmul(const double* x, const double* y, long n, double* out) {
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n;
+       i += (long)gridDim.x * blockDim.x) {
+    out[i] = soft_mul(x[i], y[i]);
+    out[n + i] = __dmul_rn(x[i], y[i]);
+    out[2 * n + i] = soft_twice(x[i]);
+  }
+}
+
+LevelH level_h(const Hier& H, double k = 0.01, double cL = 4.0) {
   LevelH lh;
   for (int l = 0; l < NRD_MAX_LEVELS; l++)
     for (int d = 0; d < 3; d++) {
@@ -1037,18 +1038,26 @@ LevelH level_h(const Hier& H, double k = 0.01, double beta = 0.0) {
       lh.rh[l][d] = 1.0 / h;
       lh.h3[l][d] = 3.0 * h;
       lh.kh[l][d] = k / h;
-      lh.kh5[l][d] = 1.25 * k / h;
-      lh.bh2[l][d] = beta / (h * h);
-      lh.h12[l][d] = 12.0 * h;
-      lh.khs[l][d] = kP52 * (k / h);
-      lh.kh5s[l][d] = kP32 * (1.25 * k / h);
+      lh.c1[l][d] = 1.0 / (12.0 * h * h);
+      lh.cLh[l][d] = 0.5 * cL * h;
+      lh.cT[l][d] = kP52 * (k / (h * h));
     }
   return lh;
 }
 
+// the constants of the faces in the soft window (softfp.h), so that products
+// with in-window cell values stay normal
+bool soft_constants(const Hier& H, const LevelH& lh) {
+  auto in = [](double x) { return x >= 0x1p-64 && x < 0x1p64; };
+  for (int l = 0; l < H.L; l++)
+    for (int d = 0; d < 3; d++)
+      if (!in(lh.c1[l][d]) || !in(lh.cLh[l][d]) || !in(lh.cT[l][d])) return false;
+  return true;
+}
+
 template <int MODE, int TX, int TY, int TZ>
 size_t stencil_smem() {
-  if (MODE == ST_LINC || MODE == ST_RESC) return 0;   // cells and faces from global memory
+  if (MODE == ST_LINC || MODE == ST_LINZC || MODE == ST_RESC) return 0;   // cells and faces from global memory
   constexpr int NH = (TX + 2) * (TY + 2) * (TZ + 2);
   constexpr int NF = (TX + 1) * TY * TZ + TX * (TY + 1) * TZ + TX * TY * (TZ + 1);
   size_t d = (size_t)NH * (MODE == ST_JV ? 5 : (MODE == ST_JVF ? 2 : 3)) + 2 * (size_t)NF;
@@ -1130,38 +1139,38 @@ void launch_ghost_z(const Hier& H, const float* z, float* gz, cudaStream_t s) {
   k_ghost_z<<<blocks_for(H.G, 256), 256, 0, s>>>(H.d_gzsrc, z, gz, H.G);
 }
 
-void launch_stencil(const Hier& H, const ModelParams& mp, const float* z, const float* gz,
-                    int mode, const StencilIO& io, cudaStream_t s, const double* z3) {
+void launch_stencil(const Hier& H, const ModelParams& mp, int mode, const StencilIO& io,
+                    cudaStream_t s, const double* z3) {
   StArgs a;
   a.z3 = z3;
   a.tiles = H.d_tiles;
   a.patches = H.d_patches;
   a.mask = H.d_mask;
   a.gtype = H.d_gtype;
-  a.z = z;
-  a.gz = gz;
   a.ntiles = (int)H.tiles.size();
   a.N = H.N;
   a.G = H.G;
-  a.k = mp.k;
   a.cL = (mp.limiter == NRD_LIM_PAPER_LITERAL) ? 2.0 : 4.0;
-  a.cL2 = 0.5 * a.cL;
-  a.m15cL = -1.5 * a.cL;
   for (int f = 0; f < 6; f++) a.R[f] = mp.bc_R[f];
-  a.lh = level_h(H, mp.k, io.beta);
+  a.lh = level_h(H, mp.k, a.cL);
+  a.soft = soft_constants(H, a.lh);
   a.io = io;
-  if (mode == ST_RESIDUAL && io.pef) {
+  if (mode == ST_RESIDUAL) {
     dispatch_tile<ST_RESF>(a, H.tile_x, H.tile_y, H.tile_z, s);
     dispatch_tile_h<ST_RESC>(H, a, s);
-  } else if (mode == ST_RESIDUAL) dispatch_tile<ST_RESIDUAL>(a, H.tile_x, H.tile_y, H.tile_z, s);
-  else if (mode == ST_JV) dispatch_tile<ST_JV>(a, H.tile_x, H.tile_y, H.tile_z, s);
-  else if (mode == ST_LIN && io.pef) {
+  } else if (mode == ST_JV) {
+    dispatch_tile<ST_JV>(a, H.tile_x, H.tile_y, H.tile_z, s);
+  } else if (mode == ST_LIN) {
     dispatch_tile<ST_LINF>(a, H.tile_x, H.tile_y, H.tile_z, s);
     dispatch_tile_h<ST_LINC>(H, a, s);
-  } else if (mode == ST_LIN) dispatch_tile<ST_LIN>(a, H.tile_x, H.tile_y, H.tile_z, s);
-  else if (mode == ST_LINZ) dispatch_tile<ST_LINZ>(a, H.tile_x, H.tile_y, H.tile_z, s);
-  else if (mode == ST_JVF) dispatch_tile_h<ST_JVF>(H, a, s);
-  else dispatch_tile<ST_FD>(a, H.tile_x, H.tile_y, H.tile_z, s);
+  } else if (mode == ST_LINZ) {
+    dispatch_tile<ST_LINZF>(a, H.tile_x, H.tile_y, H.tile_z, s);
+    dispatch_tile_h<ST_LINZC>(H, a, s);
+  } else if (mode == ST_JVF) {
+    dispatch_tile_h<ST_JVF>(H, a, s);
+  } else {
+    dispatch_tile<ST_FD>(a, H.tile_x, H.tile_y, H.tile_z, s);
+  }
 }
 
 void launch_reflux(const Hier& H, const StencilIO& io, int mode, cudaStream_t s) {
@@ -1171,13 +1180,11 @@ void launch_reflux(const Hier& H, const StencilIO& io, int mode, cudaStream_t s)
   a.off = H.d_rf_off;
   a.face = H.d_rf_face;
   a.g = H.d_rf_g;
-  a.patches = H.d_patches;
   a.nrf = H.nrf;
   a.N = H.N;
   a.G = H.G;
-  a.lh = level_h(H);
-  k_reflux<<<blocks_for(H.nrf, 128), 128, 0, s>>>(a, H.d_rf_level, io.cfflux, io.out, io.dt,
-                                                   io.par, io.eps, mode);
+  k_reflux<<<blocks_for(H.nrf, 128), 128, 0, s>>>(a, io.cfflux, io.out, io.dt, io.par, io.eps,
+                                                   mode);
 }
 
 void launch_jv_frozen(const Hier& H, const ModelParams& mp, const double* jc, const double* cc,
@@ -1187,7 +1194,7 @@ void launch_jv_frozen(const Hier& H, const ModelParams& mp, const double* jc, co
   StencilIO q = io;
   q.jc = const_cast<double*>(jc);
   q.cc = const_cast<double*>(cc);
-  launch_stencil(H, mp, nullptr, nullptr, ST_JVF, q, s);
+  launch_stencil(H, mp, ST_JVF, q, s, nullptr);
 }
 
 void launch_tag(const Hier& H, const double* E, const double* gE, double thr_c, double thr_g,
@@ -1211,6 +1218,15 @@ extern "C" int nrd_check_fastmath(const double* x, int64_t n, double* out, cudaS
   if (n == 0) return NRD_OK;
   const int grid = (int)std::min<long>(152L * 8, (n + 255) / 256);
   k_check_fastmath<<<grid, 256, 0, s>>>(x, n, out);
+  return cudaGetLastError() == cudaSuccess ? NRD_OK : NRD_ECUDA;
+}
+
+extern "C" int nrd_check_softmul(const double* x, const double* y, int64_t n, double* out,
+                                 cudaStream_t s) {
+  if (!x || !y || !out || n < 0) return NRD_EINVAL;
+  if (n == 0) return NRD_OK;
+  const int grid = (int)std::min<long>(152L * 8, (n + 255) / 256);
+  k_check_softmul<<<grid, 256, 0, s>>>(x, y, n, out);
   return cudaGetLastError() == cudaSuccess ? NRD_OK : NRD_ECUDA;
 }
 

@@ -2,9 +2,10 @@
 // product), at the state of the last linearisation.  Gather form, no atomics,
 // deterministic:
 //   1. face adjoints   lambda_f = sum over the cells whose balance uses face f
-//                      of (+-1/h) w_cell, including the coarse cell of a
-//                      coarse-fine face through flux matching (1/4 of the fine
-//                      face, on the coarse side);
+//                      of +-w_cell (the flux partials are over h), including
+//                      the coarse cell of a coarse-fine face through flux
+//                      matching (1/8: a quarter of the fine face over twice
+//                      the fine h);
 //   2. ghost adjoints  gamma_g = the ghost side's flux partials times lambda;
 //   3. cell gather     (J^T w)_c = a0 w_c - dt (sum of the cell's own face
 //                      partials times lambda + the ghost adjoints of every
@@ -39,7 +40,6 @@ struct VjpArgs {
   double* dz;          // [N] or null
   double a0, dt;
   int N, G, ntiles, tx, ty, tz;
-  double rh[NRD_MAX_LEVELS][3];
 };
 
 __device__ __forceinline__ bool leaf(const uint8_t* mask, int c) {
@@ -65,19 +65,18 @@ __global__ void k_vjp_faces(VjpArgs a) {
       const bool lf = leaf(a.mask, idx);
       const double wE = a.w[idx], wT = a.w[N + idx];
       for (int d = 0; d < 3; d++) {
-        const double rh = a.rh[P.level][d];
         if (loc[d] > 0) {
           // interior face between a = idx - st (low) and b = idx (high)
           const int ia = idx - st[d];
           const uint8_t ma = a.mask[ia];
           double lE = 0.0, lT = 0.0;
           if (leaf(a.mask, ia) && !(ma & (2 << (2 * d + 1)))) {
-            lE += a.w[ia] * rh;
-            lT += a.w[N + ia] * rh;
+            lE += a.w[ia];
+            lT += a.w[N + ia];
           }
           if (lf && !(m & (2 << (2 * d)))) {
-            lE -= wE * rh;
-            lT -= wT * rh;
+            lE -= wE;
+            lT -= wT;
           }
           const long slot = (long)d * N + idx;
           a.lam[slot] = lE;
@@ -96,14 +95,13 @@ __global__ void k_vjp_faces(VjpArgs a) {
             // this cell is the low side of its high face (sd = 1), the high
             // side of its low face (sd = 0)
             const double sg = sd ? 1.0 : -1.0;
-            lE += sg * wE * rh;
-            lT += sg * wT * rh;
+            lE += sg * wE;
+            lT += sg * wT;
             if (ty == GT_CF) {
               // the coarse cell across the face takes 1/4 of this fine flux
               const int C = a.gzsrc[g];
-              const double rhc = a.rh[P.level - 1][d];
-              lE -= sg * 0.25 * a.w[C] * rhc;
-              lT -= sg * 0.25 * a.w[N + C] * rhc;
+              lE -= sg * 0.125 * a.w[C];
+              lT -= sg * 0.125 * a.w[N + C];
             }
           }
           a.lam[slot] = lE;
@@ -241,8 +239,6 @@ void launch_vjp(const Hier& H, const double* jc, const double* cc, const float* 
   a.tx = H.tile_x;
   a.ty = H.tile_y;
   a.tz = H.tile_z;
-  for (int l = 0; l < NRD_MAX_LEVELS; l++)
-    for (int d = 0; d < 3; d++) a.rh[l][d] = (l < H.L) ? 1.0 / H.lev[l].h[d] : 1.0;
   const int nt = std::max(1, (int)H.tiles.size());
   k_vjp_faces<<<nt, 256, 0, s>>>(a);
   int gb = (int)std::min(152L * 8, (H.G + 255L) / 256);

@@ -124,11 +124,13 @@ void hier_free(Hier& H);
 
 // Kernel launchers (k_stencil.cu)
 // stencil modes; ST_JVF applies the Jacobian frozen by ST_LIN (jc, cc) to v;
-// ST_LINZ is ST_LIN that also forms the partials with respect to z^3
-// ST_LINF / ST_LINC (ST_RESF / ST_RESC): ST_LIN (ST_RESIDUAL) in two launches,
-// every face once (face fluxes to StencilIO::pef), then the cell balance from them
+// ST_LINZ is ST_LIN that also forms the partials with respect to z^3.
+// The residual and the linearisation run as two launches (ST_RESF / ST_RESC,
+// ST_LINF / ST_LINC, ST_LINZF / ST_LINZC): every face once, its flux over h to
+// StencilIO::pef, then the cell balance from them.  Every face flux and flux
+// partial is kept divided by h (its share of a cell's divergence).
 enum { ST_RESIDUAL = 0, ST_JV = 1, ST_FD = 2, ST_LIN = 3, ST_JVF = 4, ST_LINZ = 5, ST_LINF = 6,
-       ST_LINC = 7, ST_RESF = 8, ST_RESC = 9 };
+       ST_LINC = 7, ST_RESF = 8, ST_RESC = 9, ST_LINZF = 10, ST_LINZC = 11 };
 struct StencilIO {
   const double* u;      // state (E then T)
   const double* v;      // direction (JV, FD)
@@ -150,14 +152,14 @@ struct StencilIO {
   double* p2;           // [3][N] P2 data (FP64 V-cycle), or
   float* p2f;           //   FP32 (FP32 V-cycle)
   const double* par;    // device [a0, dt, beta] overriding a0, dt, beta (or null)
-  double* pef = nullptr;  // [2][3N+G] face fluxes: ST_LIN / ST_RESIDUAL run split when set
+  double* pef = nullptr;  // [2][3N+G] face fluxes over h (residual, linearisation)
 };
 void launch_ghost_fill(const Hier& H, const ModelParams& mp, const float* z, const double* u,
                        double* g, int nonlinear, cudaStream_t s);
 void launch_ghost_z(const Hier& H, const float* z, float* gz, cudaStream_t s);
-// z3 (optional): z^3 in FP64 for the cells followed by the ghosts (N + G)
-void launch_stencil(const Hier& H, const ModelParams& mp, const float* z, const float* gz,
-                    int mode, const StencilIO& io, cudaStream_t s, const double* z3 = nullptr);
+// z3: z^3 in FP64 for the cells followed by the ghosts (N + G); not read by ST_JVF
+void launch_stencil(const Hier& H, const ModelParams& mp, int mode, const StencilIO& io,
+                    cudaStream_t s, const double* z3);
 // z3[c] = z[c]^3 (cells), z3[N + g] = gz[g]^3 (ghosts), in FP64
 void launch_cube(const Hier& H, const float* z, const float* gz, double* z3, cudaStream_t s);
 void launch_reflux(const Hier& H, const StencilIO& io, int mode, cudaStream_t s);

@@ -30,7 +30,7 @@ EXPORTED = [
     "nrd_step", "nrd_step_begin", "nrd_step_end", "nrd_tag", "nrd_regrid_boxes", "nrd_transfer", "nrd_time_derivative", "nrd_predict", "nrd_lte", "nrd_dt_control",
     "nrd_autotune", "nrd_autotune_sweeps", "nrd_wdot_noalloc", "nrd_measure_peaks",
     "nrd_measure_fp64_ops",
-    "nrd_check_fastmath", "nrd_check_narrow",
+    "nrd_check_fastmath", "nrd_check_narrow", "nrd_check_softmul",
     "nrd_timing_enable",
     "nrd_timing_read",
 ]
@@ -121,6 +121,7 @@ def load(path: str = _LIBPATH):
         "nrd_measure_fp64_ops": (c_int, [P(c_dbl), vp]),
         "nrd_check_fastmath": (c_int, [dp, ctypes.c_int64, dp, vp]),
         "nrd_check_narrow": (c_int, [dp, ctypes.c_int64, fp, vp]),
+        "nrd_check_softmul": (c_int, [dp, dp, ctypes.c_int64, dp, vp]),
         "nrd_timing_enable": (c_int, [vp, c_int]),
         "nrd_timing_read": (c_int, [vp, c_int, P(c_dbl), P(ctypes.c_int64)]),
     }
@@ -195,6 +196,16 @@ def check_narrow(x):
                                  _stream())
     if rc != OK:
         raise NrdError(rc, "nrd_check_narrow failed")
+    return out
+
+
+def check_softmul(x, y):
+    """[integer-pipe x y, __dmul_rn(x, y), integer-pipe 2 x] (nrd_check_softmul)."""
+    out = torch.empty(3, x.numel(), dtype=torch.float64, device=x.device)
+    rc = load().nrd_check_softmul(_ptr(x, torch.float64), _ptr(y, torch.float64), x.numel(),
+                                  _ptr(out, torch.float64), _stream())
+    if rc != OK:
+        raise NrdError(rc, "nrd_check_softmul failed")
     return out
 
 
