@@ -400,12 +400,13 @@ int nrd_check_fastmath(const double* x, int64_t n, double* out, cudaStream_t str
  * Asynchronous.  Errors: NRD_EINVAL (null pointer, n < 0), NRD_ECUDA. */
 int nrd_check_narrow(const double* x, int64_t n, float* out, cudaStream_t stream);
 
-/* Check of the FP64 products the stencils form on the integer pipe (no
- * counterpart in the paper): for n pairs of doubles x, y (device), out
- * (device, 3n doubles) receives the integer-instruction product x y, CUDA's
- * __dmul_rn of them, and the exponent-increment form of 2 x.  The first two
- * are bit-identical where x, y and x y are each zero or normal, the third is
- * exact where x is zero or normal and 2 x finite.
+/* Check of the FP64 products the stencils form on the integer pipe
+ * (no counterpart in the paper): for n pairs of doubles x, y (device), out
+ * (device, 4n doubles) receives the integer-instruction product x y, CUDA's
+ * __dmul_rn of them, the exponent-increment form of 2 x, and the product with
+ * a native fallback.  The first two are bit-identical where x, y and x y are
+ * each zero or normal, the third is exact where x is zero or normal and 2 x
+ * finite, the fourth is bit-identical to the second for all inputs.
  * Asynchronous.  Errors: NRD_EINVAL (null pointer, n < 0), NRD_ECUDA. */
 int nrd_check_softmul(const double* x, const double* y, int64_t n, double* out,
                       cudaStream_t stream);

@@ -85,11 +85,12 @@ void set_model(nrd_ctx* c) {
 
 void free_fields(nrd_ctx* c) {
   auto F = [](void* p) { if (p) cudaFree(p); };
-  F(c->d_z); F(c->d_gz); F(c->d_gu); F(c->d_gv); F(c->d_cf); F(c->d_tmp); F(c->d_jc); F(c->d_pef); F(c->d_cc);
-  F(c->d_lam); F(c->d_gam); F(c->d_z3);
+  F(c->d_z); F(c->d_gz); F(c->d_gu); F(c->d_gv); F(c->d_cf); F(c->d_tmp); F(c->jac.jc); F(c->d_pef);
+  F(c->d_gam); F(c->d_z3);
+  c->jac = Jac();
   c->d_z3 = nullptr;
   c->d_z = nullptr; c->d_gz = nullptr; c->d_gu = nullptr; c->d_gv = nullptr; c->d_cf = nullptr;
-  c->d_tmp = nullptr; c->d_jc = nullptr; c->d_pef = nullptr; c->d_cc = nullptr; c->d_lam = nullptr; c->d_gam = nullptr;
+  c->d_tmp = nullptr; c->d_pef = nullptr; c->d_gam = nullptr;
   c->lin_ready = false;
   reducer_free(c->R);
   if (c->pc) pc_free(c->pc);
@@ -133,9 +134,8 @@ int ctx_linearise(nrd_ctx* c, const double* u, const double* b, double a0, doubl
   io.dt = dt;
   io.out = F;
   io.cfflux = c->d_cf;
-  io.jc = c->d_jc;
+  io.jac = c->jac;
   io.craw = pc_craw(c->pc);
-  io.cc = c->d_cc;
   io.beta = dt / a0;
   io.par = par;
   pc_lin_targets(c->pc, &io.a32, &io.a64, &io.p2, &io.p2f);
@@ -170,8 +170,9 @@ int ctx_jv(nrd_ctx* c, const double* u, const double* v, const double* b, const 
     io.par = par;
     io.out = Jv;
     io.cfflux = c->d_cf;
+    io.jac = c->jac;
     c->timer.begin(NRD_TK_JV, s);
-    launch_jv_frozen(H, c->mp, c->d_jc, c->d_cc, io, s);
+    launch_jv_frozen(H, io, s);
     c->timer.end(NRD_TK_JV, s);
     launch_reflux(H, io, ST_JV, s);
     return check_launch(c);
@@ -329,10 +330,8 @@ int nrd_set_hierarchy(nrd_ctx* c, int nlevels, const int* nboxes, const int* box
             cudaMalloc(&c->d_gv, 2 * (G ? G : 1) * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&c->d_cf, 2 * (G ? G : 1) * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&c->d_tmp, 2 * N * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&c->d_jc, 6 * (3 * N + G) * sizeof(double)) == cudaSuccess &&
+            cudaMalloc(&c->jac.jc, (23 * N + 6 * G) * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&c->d_pef, 2 * (3 * N + G) * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&c->d_cc, 3 * N * sizeof(double)) == cudaSuccess &&
-            cudaMalloc(&c->d_lam, 2 * (3 * N + G) * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&c->d_gam, 3 * (G ? G : 1) * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&c->d_z3, (N + G) * sizeof(double)) == cudaSuccess &&
             reducer_init(c->R, (int)N) == NRD_OK;
@@ -341,6 +340,8 @@ int nrd_set_hierarchy(nrd_ctx* c, int nlevels, const int* nboxes, const int* box
     hier_free(c->H);
     return fail(c, NRD_ENOMEM, "device allocation failed");
   }
+  c->jac.cen = c->jac.jc + 6 * (3 * N + G);
+  c->jac.cZ = c->jac.cen + 4 * N;
   cudaMemset(c->d_cf, 0, 2 * (G ? G : 1) * sizeof(double));
   rc = pc_alloc(&c->pc, H, c->p, err);
   if (rc != NRD_OK) {
@@ -441,7 +442,7 @@ int nrd_vjp(nrd_ctx* c, const double* w, double a0, double dt, double* JTw, doub
   if (!c->lin_ready) return fail(c, NRD_ESTATE, "nrd_vjp needs nrd_linearise first");
   if (dz && !c->lin_dz)
     return fail(c, NRD_ESTATE, "dz needs the material partials: call nrd_linearise first");
-  launch_vjp(c->H, c->d_jc, c->d_cc, c->d_z, w, c->d_lam, c->d_gam, a0, dt, JTw, dz, s);
+  launch_vjp(c->H, c->jac, c->d_z, w, c->d_gam, a0, dt, JTw, dz, s);
   return check_launch(c);
 }
 

@@ -201,8 +201,9 @@ __device__ __forceinline__ float narrow_rn(double x) {
 //   Phi_T / h = T25 dT with T25 = cT Ts^(5/2) (= D_T / h^2).
 // 13 FP64 instructions and 12 products; the products go to the integer pipe
 // where SOFT (the same bits, see softfp.h).  Both pipes then take about the
-// same time.  Measured at 256^3 (8x8x8 tiles): the linearisation's face launch
-// @LINF@, the residual's @RESF@.
+// same time.  Measured at 256^3 (8x8x8 tiles), against the plain formulas on the
+// FP64 pipe alone (45 and 26 instructions a face): the linearisation's face
+// launch 4.25 -> 2.16 ms, the residual's 2.66 -> 1.37 ms.
 struct FaceCore {
   double Ts, dE, S, r, Q, X, lt, PE, y, dT, T25, PT;
 };
@@ -338,22 +339,32 @@ __device__ __forceinline__ void put_scaled(const StencilIO& io, long NS, long sl
   }
 }
 
-// The linearisation's cell outputs: F from cell_balance, the coupling
-// partials and the P2 data.
+// the faces' part of a cell's own Jacobian entries
+struct OwnSum {
+  double EE, ET, TT;
+};
+
+// The linearisation's cell outputs: F from cell_balance, the own entries of
+// the frozen Jacobian and the P2 data.
 template <bool DZ, bool SOFT>
 __device__ __forceinline__ void lin_cell(const StencilIO& io, int N, int idx, double a0v,
                                          double dtv, double betav, float betaf, double E,
-                                         double T, double z3, double divE, double divT) {
+                                         double T, double z3, double divE, double divT,
+                                         const OwnSum& own) {
   using M = Mul<SOFT>;
   double FE, FT, rT, sig;
   cell_balance<SOFT>(a0v, dtv, E, T, z3, io.b[idx], io.b[N + idx], divE, divT, FE, FT, rT, sig);
   io.out[idx] = FE;
   io.out[N + idx] = FT;
   const double T2 = M::pos(T, T), T3 = M::pos(T2, T);
-  // coupling tangent dc = cE vE + cT vT
-  io.cc[idx] = -sig;
-  io.cc[N + idx] = M::pos(sig, fma(M::pos(3.0, E), rT, T3));
-  if (DZ) io.cc[2L * N + idx] = (T2 * T2 - E) * rT * rT * rT;   // d coupling / d z^3
+  // coupling tangent dc = -sig vE + cT vT, with the own entries of the faces
+  const double cT = M::pos(sig, fma(M::pos(3.0, E), rT, T3));
+  double* cen = io.jac.cen;
+  cen[idx] = own.EE - sig;
+  cen[N + idx] = own.ET + cT;
+  cen[2L * N + idx] = own.TT - cT;
+  cen[3L * N + idx] = sig;
+  if (DZ) io.jac.cZ[idx] = (T2 * T2 - E) * rT * rT * rT;   // d coupling / d z^3
   // P2 of Sec. 4.2 at this iterate: [[1 + sb, -sbt], [-sb, 1 + sbt]]
   // (det = (1 + sb)(1 + sbt) - sbt sb = 1 + sb + sbt), in the
   // preconditioner's precision
@@ -375,9 +386,8 @@ template <bool DZ>
 __device__ __forceinline__ void lin_cell_covered(const StencilIO& io, int N, int idx) {
   io.out[idx] = 0.0;
   io.out[N + idx] = 0.0;
-  io.cc[idx] = 0.0;
-  io.cc[N + idx] = 0.0;
-  if (DZ) io.cc[2L * N + idx] = 0.0;
+  for (int q = 0; q < 4; q++) io.jac.cen[(long)q * N + idx] = 0.0;
+  if (DZ) io.jac.cZ[idx] = 0.0;
   if (io.p2f) {
     io.p2f[idx] = 0.0f;
     io.p2f[N + idx] = 0.0f;
@@ -389,6 +399,21 @@ __device__ __forceinline__ void lin_cell_covered(const StencilIO& io, int N, int
   }
 }
 
+// Resident blocks per SM the split forms' launches are compiled for.  They
+// need warps to cover the latency of their loads and integer products more
+// than registers.  Measured at 256^3 (us; the compiler's own choice -> this):
+// linearisation faces 2277 -> 2159 (4), cells 1326 -> 1247 (4), residual
+// faces 1408 -> 1372 (8), cells on an odd box 40.6 -> 39.7 (5); the cells of
+// three levels of ragged patches 603 -> 437 (4).
+constexpr int min_blocks(int mode) {
+  switch (mode) {
+    case ST_LINF: case ST_LINZF: case ST_LINC: case ST_LINZC: return 4;
+    case ST_RESF: return 8;
+    case ST_RESC: return 5;
+    default: return 0;   // no bound
+  }
+}
+
 // CMP: the cell loops (and the fused forms' face loop) run over the cells of
 // a tile inside its patch only, with index arithmetic in the tile's runtime
 // extent; used where the hierarchy has tiles narrower than the tile shape
@@ -397,7 +422,7 @@ __device__ __forceinline__ void lin_cell_covered(const StencilIO& io, int N, int
 // compile-time shape (fewer registers: the form for hierarchies without
 // such tiles).
 template <int MODE, int TX, int TY, int TZ, bool CMP = false>
-__global__ void __launch_bounds__(256) k_stencil(StArgs A) {
+__global__ void __launch_bounds__(256, min_blocks(MODE)) k_stencil(StArgs A) {
   constexpr int HX = TX + 2, HY = TY + 2, HZ = TZ + 2;
   constexpr int NH = HX * HY * HZ;
   constexpr int NFX = (TX + 1) * TY * TZ, NFY = TX * (TY + 1) * TZ, NFZ = TX * TY * (TZ + 1);
@@ -408,7 +433,6 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
   constexpr bool FACES = LIN || MODE == ST_RESF;    // split forms: faces only
   constexpr bool CELLS = LINC || MODE == ST_RESC;   // split forms: cells only
   constexpr bool DZ = (MODE == ST_LINZF || MODE == ST_LINZC);   // also the d/dz^3 partials
-  constexpr bool JVF = (MODE == ST_JVF);       // frozen-Jacobian Jv: sE, sT hold v
   extern __shared__ double smem[];
   double* sE = smem;
   double* sT = sE + NH;
@@ -420,7 +444,7 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
   double* fyT = fyE + NFY;
   double* fzE = fyT + NFY;
   double* fzT = fzE + NFZ;
-  double* sZ = fzT + NFZ;                     // z^3 of the halo cells
+  double* sZ = FACES ? fxE : fzT + NFZ;       // z^3 of the halo cells
 
   const int N = A.N, G = A.G;
   const long NS = 3L * N + G;                  // face slots per coefficient array
@@ -499,12 +523,25 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
         const double divT = (pick(m & 4, pT[xh]) - pick(m & 2, pT[xl])) +
                             (pick(m & 16, pT[yh]) - pick(m & 8, pT[yl])) +
                             (pick(m & 64, pT[zh]) - pick(m & 32, pT[zl]));
+        // own entries: its side's partials of its six faces
+        OwnSum own = {0.0, 0.0, 0.0};
+        if (LINC) {
+          const double* jc = io.jac.jc;
+          auto sum = [&](const double* a, const double* b) {
+            return (pick(m & 4, a[xh]) - pick(m & 2, b[xl])) +
+                   (pick(m & 16, a[yh]) - pick(m & 8, b[yl])) +
+                   (pick(m & 64, a[zh]) - pick(m & 32, b[zl]));
+          };
+          own.EE = sum(jc, jc + NS);
+          own.ET = sum(jc + 2 * NS, jc + 2 * NS);
+          own.TT = sum(jc + 3 * NS, jc + 4 * NS);
+        }
         const double E = io.u[idx], T = io.u[N + idx];
         const double z3c = A.z3[idx];
         auto cell = [&](auto soft) {
           constexpr bool SOFT = decltype(soft)::value;
           if (LINC) {
-            lin_cell<DZ, SOFT>(io, N, idx, a0v, dtv, betav, betaf, E, T, z3c, divE, divT);
+            lin_cell<DZ, SOFT>(io, N, idx, a0v, dtv, betav, betaf, E, T, z3c, divE, divT, own);
           } else {
             double FE, FT, rT, sig;
             cell_balance<SOFT>(a0v, dtv, E, T, z3c, io.b[idx], io.b[N + idx], divE, divT, FE, FT,
@@ -530,22 +567,6 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
       if (i > nx || j > ny || k > tile.k1) continue;
       double e, tt, ve = 0.0, vt = 0.0;
       double z = 0.0;
-      if (JVF) {
-        if (!ox && !oy && !oz) {
-          int idx = P.off + i + nx * (j + ny * k);
-          e = io.v[idx];
-          tt = io.v[N + idx];
-        } else {
-          int f = ox ? (ox < 0 ? 0 : 1) : (oy ? (oy < 0 ? 2 : 3) : (oz < 0 ? 4 : 5));
-          int a = ox ? j : (oy ? k : i), b = ox ? k : (oy ? i : j);
-          int gi = P.goff + P.fo[f] + a + P.n[(f / 2 + 1) % 3] * b;
-          e = io.gv[gi];
-          tt = io.gv[G + gi];
-        }
-        sE[hh] = e;
-        sT[hh] = tt;
-        continue;
-      }
       if (!ox && !oy && !oz) {
         int idx = P.off + i + nx * (j + ny * k);
         e = io.u[idx];
@@ -686,25 +707,11 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
       } else {
         fslot = (long)dir * N + P.off + i + (long)nx * (j + (long)ny * k);
       }
-      if (JVF) {
-        // tangent flux = stored partials times the direction (sE, sT hold v)
-        if (gt == GT_ROBIN) {
-          const int hc = (pos == 0) ? hb : ha;
-          PE = io.jc[fslot] * sE[hc] + io.jc[NS + fslot] * sT[hc];
-        } else if (gt != GT_NEUMANN) {
-          PE = io.jc[fslot] * sE[ha] + io.jc[NS + fslot] * sE[hb] +
-               io.jc[2 * NS + fslot] * (sT[ha] + sT[hb]);
-          PT = io.jc[3 * NS + fslot] * sT[ha] + io.jc[4 * NS + fslot] * sT[hb];
-          if (gt == GT_CF) {
-            io.cfflux[gi] = PE;
-            io.cfflux[G + gi] = PT;
-          }
-        }
-      } else if (gt == GT_NEUMANN) {
+      if (gt == GT_NEUMANN) {
         PE = 0.0;
         PT = 0.0;
         if (LIN) {
-          for (int q = 0; q < 6; q++) io.jc[q * NS + fslot] = 0.0;
+          for (int q = 0; q < 6; q++) io.jac.jc[q * NS + fslot] = 0.0;
           put_scaled(io, NS, fslot, 0.0, 0.0);
         }
       } else if (gt == GT_ROBIN) {
@@ -718,18 +725,18 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
           PE = rh * robin_flux(sE[hc], sT[hc], sZ[hc], h, A.R[ff], s);
         }
         if (LIN) {
-          // dPhi/dE_c and dPhi/dT_c over h in slots 0 and 1; raw P1 slot holds D_b
+          // dPhi/dE_c and dPhi/dT_c over h, the same on both sides (only the
+          // cell's own is read); raw P1 slot holds D_b
           double Ec = sE[hc], Tc = sT[hc], zc = sZ[hc];
           double Db = Tc * Tc * Tc / (3.0 * zc);
           double qd = 4.0 * Db + h;
           double rq = 1.0 / qd;
           double m = 2.0 * Ec - 8.0 * A.R[ff];
-          io.jc[fslot] = rh * (-(double)s * 2.0 * Db * rq);
-          io.jc[NS + fslot] = -(double)s * (Tc * Tc / zc) * m * rq * rq;
-          io.jc[2 * NS + fslot] = 0.0;
-          io.jc[3 * NS + fslot] = 0.0;
-          io.jc[4 * NS + fslot] = 0.0;
-          if (DZ) io.jc[5 * NS + fslot] = (double)s * m * rq * rq * Db / zc;  // d Phi / d z_c^3
+          double* jc = io.jac.jc + fslot;
+          jc[0] = jc[NS] = rh * (-(double)s * 2.0 * Db * rq);
+          jc[2 * NS] = -(double)s * (Tc * Tc / zc) * m * rq * rq;
+          jc[3 * NS] = jc[4 * NS] = 0.0;
+          if (DZ) jc[5 * NS] = (double)s * m * rq * rq * Db / zc;  // d Phi / d z_c^3
           io.craw[fslot] = Db;
           io.craw[NS + fslot] = 0.0;
           put_scaled(io, NS, fslot, betav * 2.0 * Db * rq / h, 0.0);
@@ -747,12 +754,13 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
                                      DZ);
           PE = L.PE;
           PT = L.PT;
-          io.jc[fslot] = L.aEa;
-          io.jc[NS + fslot] = L.aEb;
-          io.jc[2 * NS + fslot] = L.aT;
-          io.jc[3 * NS + fslot] = L.bTa;
-          io.jc[4 * NS + fslot] = L.bTb;
-          if (DZ) io.jc[5 * NS + fslot] = L.aZ;
+          double* jc = io.jac.jc + fslot;
+          jc[0] = L.aEa;
+          jc[NS] = L.aEb;
+          jc[2 * NS] = L.aT;
+          jc[3 * NS] = L.bTa;
+          jc[4 * NS] = L.bTb;
+          if (DZ) jc[5 * NS] = L.aZ;
           // only the scaled P1 coefficients beta D / h^2: the coarsening
           // averages them (raw values are kept for Robin faces alone)
           if (io.a32) {
@@ -815,11 +823,7 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
       int hc = (ci + 1) + HX * ((cj + 1) + HY * (ck + 1));
       double E = sE[hc], T = sT[hc], z = sZ[hc];
       double T2 = T * T, T3 = T2 * T;
-      if (JVF) {
-        const double dc = io.cc[idx] * E + io.cc[N + idx] * T;
-        io.out[idx] = a0v * E - dtv * (divE + dc);
-        io.out[N + idx] = a0v * T - dtv * (divT - dc);
-      } else if (MODE == ST_JV) {
+      if (MODE == ST_JV) {
         double rT = 1.0 / T;
         double sig = z * rT * rT * rT;
         double vE = svE[hc], vT = svT[hc];
@@ -836,6 +840,117 @@ __global__ void __launch_bounds__(256) k_stencil(StArgs A) {
       }
     }
     __syncthreads();
+  }
+}
+
+struct JvArgs {
+  const TileDev* tiles;
+  const PatchDev* patches;
+  const uint8_t* mask;
+  const uint8_t* gtype;
+  int N, G, tx, ty;
+  Jac jac;
+  const double* v;
+  const double* gv;
+  double* out;
+  double* cf;
+  double a0, dt;
+  const double* par;
+};
+
+// Frozen Jv: out = a0 v - dt L v, one row sum per cell and field (26 FP64
+// instructions) over the 19 coefficients of the cell; fine-side coarse-fine
+// fluxes to cf for flux matching.  One tile of the stencil list per block.
+// In flux form (each face's two tangent fluxes, then the divergence) a cell
+// took 40 FP64 instructions and the kernel was bound by the FP64 pipe; the
+// rows move 9% more bytes.  Its four plain products run on the integer pipe.
+// At 256^3: 1.30 -> 0.70 ms (six blocks per SM; the compiler's own choice of
+// three 0.76), 0.69 of the FP64 issue rate being the bound left.
+__global__ void __launch_bounds__(256, 6) k_jv_frozen(JvArgs A) {
+  const int N = A.N, G = A.G;
+  double a0 = A.a0, dt = A.dt;
+  if (A.par) {
+    a0 = A.par[0];
+    dt = A.par[1];
+  }
+  const TileDev tile = A.tiles[blockIdx.x];
+  const PatchDev P = A.patches[tile.patch];
+  const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
+  // the tile's extent inside its patch: no lane idles on a cell outside it
+  const int ex = min(A.tx, nx - tile.i0), ey = min(A.ty, ny - tile.j0);
+  const int nc = ex * ey * (tile.k1 - tile.k0);
+  const long s2 = (long)nx * ny;
+  const Jac& J = A.jac;
+  for (int c = threadIdx.x; c < nc; c += blockDim.x) {
+    const int r = c / ex, i = tile.i0 + c - r * ex;
+    const int rk = r / ey, j = tile.j0 + r - rk * ey, k = tile.k0 + rk;
+    const long idx = P.off + i + nx * (j + (long)ny * k);
+    const uint8_t m = A.mask[idx];
+    if (m & MASK_COVERED) {
+      A.out[idx] = 0.0;
+      A.out[N + idx] = 0.0;
+      continue;
+    }
+    const double* vE = A.v;
+    const double* vT = A.v + N;
+    const double vEc = vE[idx], vTc = vT[idx];
+    // the four plain products on the integer pipe (bit-identical)
+    double LE = fma(J.cen[N + idx], vTc, soft_mul_any(J.cen[idx], vEc));
+    double LT = fma(J.cen[3L * N + idx], vEc, soft_mul_any(J.cen[2L * N + idx], vTc));
+    const bool inner = i > 0 && i < nx - 1 && j > 0 && j < ny - 1 && k > 0 && k < nz - 1;
+    const long NS = 3L * N + G;
+    if (inner && m == 0) {
+      const long st[3] = {1, nx, s2};
+#pragma unroll
+      for (int d = 0; d < 3; d++) {
+        const long lo = idx - st[d], hi = idx + st[d];
+        const double* jl = J.jc + (long)d * N + idx;   // the low face's slots
+        const double* jh = jl + st[d];                 // the high face's
+        const double tl = vT[lo], th = vT[hi];
+        LE = fma(-jl[0], vE[lo], LE);
+        LE = fma(-jl[2 * NS], tl, LE);
+        LT = fma(-jl[3 * NS], tl, LT);
+        LE = fma(jh[NS], vE[hi], LE);
+        LE = fma(jh[2 * NS], th, LE);
+        LT = fma(jh[4 * NS], th, LT);
+      }
+    } else {
+      const int pos[3] = {i, j, k};
+#pragma unroll
+      for (int f = 0; f < 6; f++) {
+        if (m & (2 << f)) continue;   // flux matching
+        const int d = f >> 1, hi = f & 1;
+        const long st = (d == 0) ? 1L : (d == 1 ? (long)nx : s2);
+        double nE, nT;
+        const double* jf;
+        uint8_t gt = GT_SIBLING;
+        int g = 0;
+        if (pos[d] != (hi ? P.n[d] - 1 : 0)) {
+          const long n = hi ? idx + st : idx - st;
+          jf = J.jc + (long)d * N + (hi ? n : idx);
+          nE = vE[n];
+          nT = vT[n];
+        } else {
+          g = P.goff + P.fo[f] + pos[(d + 1) % 3] + P.n[(d + 1) % 3] * pos[(d + 2) % 3];
+          gt = A.gtype[g];
+          if (gt == GT_NEUMANN || gt == GT_ROBIN) continue;   // own entries only
+          jf = J.jc + 3L * N + g;
+          nE = A.gv[g];
+          nT = A.gv[G + g];
+        }
+        LE = fma(hi ? jf[NS] : -jf[0], nE, LE);
+        LE = fma(hi ? jf[2 * NS] : -jf[2 * NS], nT, LE);
+        LT = fma(hi ? jf[4 * NS] : -jf[3 * NS], nT, LT);
+        if (gt == GT_CF) {
+          const double Ea = hi ? vEc : nE, Eb = hi ? nE : vEc;
+          const double Ta = hi ? vTc : nT, Tb = hi ? nT : vTc;
+          A.cf[g] = fma(jf[0], Ea, fma(jf[NS], Eb, jf[2 * NS] * (Ta + Tb)));
+          A.cf[G + g] = fma(jf[3 * NS], Ta, jf[4 * NS] * Tb);
+        }
+      }
+    }
+    A.out[idx] = fma(-dt, LE, soft_mul_any(a0, vEc));
+    A.out[N + idx] = fma(-dt, LT, soft_mul_any(a0, vTc));
   }
 }
 
@@ -1026,6 +1141,7 @@ __global__ void k_check_softmul(const double* x, const double* y, long n, double
     out[i] = soft_mul(x[i], y[i]);
     out[n + i] = __dmul_rn(x[i], y[i]);
     out[2 * n + i] = soft_twice(x[i]);
+    out[3 * n + i] = soft_mul_any(x[i], y[i]);
   }
 }
 
@@ -1060,7 +1176,9 @@ size_t stencil_smem() {
   if (MODE == ST_LINC || MODE == ST_LINZC || MODE == ST_RESC) return 0;   // cells and faces from global memory
   constexpr int NH = (TX + 2) * (TY + 2) * (TZ + 2);
   constexpr int NF = (TX + 1) * TY * TZ + TX * (TY + 1) * TZ + TX * TY * (TZ + 1);
-  size_t d = (size_t)NH * (MODE == ST_JV ? 5 : (MODE == ST_JVF ? 2 : 3)) + 2 * (size_t)NF;
+  // the split forms' face launches keep no fluxes in shared memory
+  const bool faces = MODE == ST_LINF || MODE == ST_LINZF || MODE == ST_RESF;
+  size_t d = (size_t)NH * (MODE == ST_JV ? 5 : 3) + (faces ? 0 : 2 * (size_t)NF);
   return d * sizeof(double);
 }
 
@@ -1166,8 +1284,6 @@ void launch_stencil(const Hier& H, const ModelParams& mp, int mode, const Stenci
   } else if (mode == ST_LINZ) {
     dispatch_tile<ST_LINZF>(a, H.tile_x, H.tile_y, H.tile_z, s);
     dispatch_tile_h<ST_LINZC>(H, a, s);
-  } else if (mode == ST_JVF) {
-    dispatch_tile_h<ST_JVF>(H, a, s);
   } else {
     dispatch_tile<ST_FD>(a, H.tile_x, H.tile_y, H.tile_z, s);
   }
@@ -1187,14 +1303,27 @@ void launch_reflux(const Hier& H, const StencilIO& io, int mode, cudaStream_t s)
                                                    mode);
 }
 
-void launch_jv_frozen(const Hier& H, const ModelParams& mp, const double* jc, const double* cc,
-                      const StencilIO& io, cudaStream_t s) {
-  // the tiled stencil in ST_JVF mode: v staged in shared memory, each face's
-  // tangent flux formed once from the stored partials
-  StencilIO q = io;
-  q.jc = const_cast<double*>(jc);
-  q.cc = const_cast<double*>(cc);
-  launch_stencil(H, mp, ST_JVF, q, s, nullptr);
+void launch_jv_frozen(const Hier& H, const StencilIO& io, cudaStream_t s) {
+  JvArgs a;
+  a.tiles = H.d_tiles;
+  a.patches = H.d_patches;
+  a.mask = H.d_mask;
+  a.gtype = H.d_gtype;
+  a.N = H.N;
+  a.G = H.G;
+  a.tx = H.tile_x;
+  a.ty = H.tile_y;
+  a.jac = io.jac;
+  a.v = io.v;
+  a.gv = io.gv;
+  a.out = io.out;
+  a.cf = io.cfflux;
+  a.a0 = io.a0;
+  a.dt = io.dt;
+  a.par = io.par;
+  const int nt = (int)H.tiles.size();
+  const int cells = H.tile_x * H.tile_y * H.tile_z;
+  k_jv_frozen<<<nt, std::min(256, cells), 0, s>>>(a);
 }
 
 void launch_tag(const Hier& H, const double* E, const double* gE, double thr_c, double thr_g,

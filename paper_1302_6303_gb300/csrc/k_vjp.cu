@@ -1,19 +1,18 @@
 // Transposed Jacobian of the residual (the adjoint / vector-Jacobian
-// product), at the state of the last linearisation.  Gather form, no atomics,
-// deterministic:
-//   1. face adjoints   lambda_f = sum over the cells whose balance uses face f
-//                      of +-w_cell (the flux partials are over h), including
-//                      the coarse cell of a coarse-fine face through flux
-//                      matching (1/8: a quarter of the fine face over twice
-//                      the fine h);
-//   2. ghost adjoints  gamma_g = the ghost side's flux partials times lambda;
-//   3. cell gather     (J^T w)_c = a0 w_c - dt (sum of the cell's own face
-//                      partials times lambda + the ghost adjoints of every
-//                      ghost that reads c, with the ghost's stencil weight +
-//                      coupling partials), and the same for d/dz.
+// product), at the state of the last linearisation.  Gather form over the rows
+// of the frozen Jacobian (Jac), no atomics, deterministic:
+//   1. ghost adjoints  gamma_g = the ghost side's flux partials times the face
+//                      adjoint lambda_g = +-w of the ghost's cell, less 1/8 of
+//                      the coarse cell's at a coarse-fine face (flux matching:
+//                      a quarter of the fine face over twice the fine h);
+//   2. cell gather     (J^T w)_c = a0 w_c - dt (the own entries, the
+//                      neighbours' coefficients for c inside the patch, the
+//                      ghost adjoints of every ghost that reads c with the
+//                      ghost's stencil weight), and the same for d/dz.
 #include <algorithm>
 
 #include "nrd_internal.h"
+#include "softfp.h"
 
 namespace {
 
@@ -30,186 +29,137 @@ struct VjpArgs {
   const double* ts_w;
   const int* tz_off;   // ghosts taking their z from a cell
   const int* tz_g;
-  const double* jc;    // [6][NS] face partials (5: d Phi_E / d z^3)
-  const double* cc;    // [3][N] coupling partials (2: d coupling / d z^3)
+  Jac jac;
   const float* z;
   const double* w;     // [2][N]
-  double* lam;         // [2][NS]
   double* gam;         // [3][G]
   double* out;         // [2][N]
   double* dz;          // [N] or null
   double a0, dt;
-  int N, G, ntiles, tx, ty, tz;
+  int N, G, tx, ty;
 };
 
-__device__ __forceinline__ bool leaf(const uint8_t* mask, int c) {
-  return !(mask[c] & MASK_COVERED);
+// adjoint of the face between cell c and its ghost g on side hi: this cell is
+// the low side of its high face; zero where flux matching or covering takes
+// the face from the cell.  The coarse cell across a coarse-fine face takes
+// a quarter of the fine flux (over its own h).
+__device__ __forceinline__ double face_adj(const VjpArgs& a, const double* w, int c, int g,
+                                           bool hi, uint8_t ty) {
+  double l = w[c];
+  if (ty == GT_CF) l -= 0.125 * w[a.gzsrc[g]];
+  return hi ? l : -l;
 }
 
-// 1. face adjoints of the low faces and boundary faces of every cell
-__global__ void k_vjp_faces(VjpArgs a) {
-  const int N = a.N, G = a.G;
-  const long NS = 3L * N + G;
-  const int nc = a.tx * a.ty * a.tz;
-  for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-    const TileDev tile = a.tiles[t];
-    const PatchDev P = a.patches[tile.patch];
-    const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-      int i = tile.i0 + c % a.tx, j = tile.j0 + (c / a.tx) % a.ty, k = tile.k0 + c / (a.tx * a.ty);
-      if (i >= nx || j >= ny || k >= tile.k1) continue;
-      const int idx = P.off + i + nx * (j + ny * k);
-      const int loc[3] = {i, j, k};
-      const int st[3] = {1, nx, nx * ny};
-      const uint8_t m = a.mask[idx];
-      const bool lf = leaf(a.mask, idx);
-      const double wE = a.w[idx], wT = a.w[N + idx];
-      for (int d = 0; d < 3; d++) {
-        if (loc[d] > 0) {
-          // interior face between a = idx - st (low) and b = idx (high)
-          const int ia = idx - st[d];
-          const uint8_t ma = a.mask[ia];
-          double lE = 0.0, lT = 0.0;
-          if (leaf(a.mask, ia) && !(ma & (2 << (2 * d + 1)))) {
-            lE += a.w[ia];
-            lT += a.w[N + ia];
-          }
-          if (lf && !(m & (2 << (2 * d)))) {
-            lE -= wE;
-            lT -= wT;
-          }
-          const long slot = (long)d * N + idx;
-          a.lam[slot] = lE;
-          a.lam[NS + slot] = lT;
-        }
-        for (int sd = 0; sd < 2; sd++) {
-          const bool at = sd ? (loc[d] == P.n[d] - 1) : (loc[d] == 0);
-          if (!at) continue;
-          const int f = 2 * d + sd;
-          const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
-          const int g = P.goff + P.fo[f] + loc[t1] + P.n[t1] * loc[t2];
-          const uint8_t ty = a.gtype[g];
-          const long slot = 3L * N + g;
-          double lE = 0.0, lT = 0.0;
-          if (ty != GT_NEUMANN && lf && !(m & (2 << f))) {
-            // this cell is the low side of its high face (sd = 1), the high
-            // side of its low face (sd = 0)
-            const double sg = sd ? 1.0 : -1.0;
-            lE += sg * wE;
-            lT += sg * wT;
-            if (ty == GT_CF) {
-              // the coarse cell across the face takes 1/4 of this fine flux
-              const int C = a.gzsrc[g];
-              lE -= sg * 0.125 * a.w[C];
-              lT -= sg * 0.125 * a.w[N + C];
-            }
-          }
-          a.lam[slot] = lE;
-          a.lam[NS + slot] = lT;
-        }
-      }
-    }
-  }
-}
-
-// 2. ghost adjoints: the ghost side's partials times the face adjoint
+// 1. ghost adjoints
 __global__ void k_vjp_ghosts(VjpArgs a) {
-  const int N = a.N, G = a.G;
-  const long NS = 3L * N + G;
+  const int N = a.N;
+  const long G = a.G;
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
     const uint8_t ty = a.gtype[g];
     double gE = 0.0, gT = 0.0, gZ = 0.0;
-    if (ty == GT_SIBLING || ty == GT_CF) {
-      const long slot = 3L * N + g;
-      const bool hi = (a.gface[g] & 7) % 2;   // ghost on the high side of the face
-      const double lE = a.lam[slot], lT = a.lam[NS + slot];
-      gE = (hi ? a.jc[NS + slot] : a.jc[slot]) * lE;
-      gT = a.jc[2 * NS + slot] * lE + (hi ? a.jc[4 * NS + slot] : a.jc[3 * NS + slot]) * lT;
-      gZ = a.jc[5 * NS + slot] * lE;
+    const int c = a.gcell[g], f = a.gface[g] & 7;
+    const uint8_t m = a.mask[c];
+    if ((ty == GT_SIBLING || ty == GT_CF) && !(m & MASK_COVERED) && !(m & (2 << f))) {
+      const bool hi = f & 1;   // ghost on the high side of the face
+      const double lE = face_adj(a, a.w, c, g, hi, ty), lT = face_adj(a, a.w + N, c, g, hi, ty);
+      const long NS = 3L * N + G;
+      const double* jf = a.jac.jc + 3L * N + g;
+      gE = (hi ? jf[NS] : jf[0]) * lE;
+      gT = jf[2 * NS] * lE + (hi ? jf[4 * NS] : jf[3 * NS]) * lT;
+      if (a.dz) gZ = jf[5 * NS] * lE;
     }
     a.gam[g] = gE;
     a.gam[G + g] = gT;
-    a.gam[2L * G + g] = gZ;
+    a.gam[2 * G + g] = gZ;
   }
 }
 
-// 3. per-cell gather
-__global__ void k_vjp_cells(VjpArgs a) {
-  const int N = a.N, G = a.G;
+// 2. per-cell gather: 26 FP64 instructions and the 19 coefficients of the rows
+// per cell (as the forward product), against three kernels with the face
+// adjoints through memory before; at 96^3 with 8 fine boxes (1.0M cells) the
+// product 134 -> 67 us.
+template <bool DZ>
+__global__ void __launch_bounds__(256, 6) k_vjp_cells(VjpArgs a) {
+  const int N = a.N;
+  const long G = a.G;
+  const TileDev tile = a.tiles[blockIdx.x];
+  const PatchDev P = a.patches[tile.patch];
+  const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
+  // the tile's extent inside its patch: no lane idles on a cell outside it
+  const int ex = min(a.tx, nx - tile.i0), ey = min(a.ty, ny - tile.j0);
+  const int nc = ex * ey * (tile.k1 - tile.k0);
+  const Jac& J = a.jac;
   const long NS = 3L * N + G;
-  const int nc = a.tx * a.ty * a.tz;
-  for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-    const TileDev tile = a.tiles[t];
-    const PatchDev P = a.patches[tile.patch];
-    const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-      int i = tile.i0 + c % a.tx, j = tile.j0 + (c / a.tx) % a.ty, k = tile.k0 + c / (a.tx * a.ty);
-      if (i >= nx || j >= ny || k >= tile.k1) continue;
-      const int idx = P.off + i + nx * (j + ny * k);
-      const uint8_t m = a.mask[idx];
-      if (m & MASK_COVERED) {
-        a.out[idx] = 0.0;
-        a.out[N + idx] = 0.0;
-        if (a.dz) a.dz[idx] = 0.0;
+  const double* wE = a.w;
+  const double* wT = a.w + N;
+  for (int q = threadIdx.x; q < nc; q += blockDim.x) {
+    const int r = q / ex, i = tile.i0 + q - r * ex;
+    const int rk = r / ey, j = tile.j0 + r - rk * ey, k = tile.k0 + rk;
+    const int idx = P.off + i + nx * (j + ny * k);
+    const uint8_t m = a.mask[idx];
+    if (m & MASK_COVERED) {
+      a.out[idx] = 0.0;
+      a.out[N + idx] = 0.0;
+      if (DZ) a.dz[idx] = 0.0;
+      continue;
+    }
+    const double wEc = wE[idx], wTc = wT[idx];
+    // the four plain products on the integer pipe (bit-identical)
+    double aE = fma(J.cen[3L * N + idx], wTc, soft_mul_any(J.cen[idx], wEc));
+    double aT = fma(J.cen[N + idx], wEc, soft_mul_any(J.cen[2L * N + idx], wTc));
+    double aZ = 0.0;
+    const int pos[3] = {i, j, k};
+#pragma unroll
+    for (int f = 0; f < 6; f++) {
+      if (m & (2 << f)) continue;   // flux matching: the neighbour is covered
+      const int d = f >> 1, hi = f & 1;
+      const int st = (d == 0) ? 1 : (d == 1 ? nx : nx * ny);
+      if (pos[d] != (hi ? P.n[d] - 1 : 0)) {
+        // the neighbour's row: its coefficient for this cell
+        const long n = hi ? idx + st : idx - st;
+        const double* jf = J.jc + (long)d * N + (hi ? n : idx);
+        const double wn = wE[n];
+        aE = fma(hi ? -jf[0] : jf[NS], wn, aE);
+        aT = fma(hi ? -jf[2 * NS] : jf[2 * NS], wn, aT);
+        aT = fma(hi ? -jf[3 * NS] : jf[4 * NS], wT[n], aT);
+        if (DZ) aZ = fma(jf[5 * NS], hi ? wEc - wn : wn - wEc, aZ);
         continue;
       }
-      const int loc[3] = {i, j, k};
-      const int st[3] = {1, nx, nx * ny};
-      double accE = 0.0, accT = 0.0, accZ = 0.0;
-      for (int d = 0; d < 3; d++) {
-        for (int sd = 0; sd < 2; sd++) {
-          const int f = 2 * d + sd;
-          if (m & (2 << f)) continue;                      // flux matching face
-          const bool bnd = sd ? (loc[d] == P.n[d] - 1) : (loc[d] == 0);
-          long slot;
-          uint8_t ty = GT_SIBLING;
-          if (!bnd) {
-            slot = (long)d * N + (sd ? idx + st[d] : idx);
-          } else {
-            const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
-            const int g = P.goff + P.fo[f] + loc[t1] + P.n[t1] * loc[t2];
-            ty = a.gtype[g];
-            slot = 3L * N + g;
-          }
-          if (ty == GT_NEUMANN) continue;
-          const double lE = a.lam[slot], lT = a.lam[NS + slot];
-          if (ty == GT_ROBIN) {
-            accE += a.jc[slot] * lE;
-            accT += a.jc[NS + slot] * lE;
-            accZ += a.jc[5 * NS + slot] * lE;
-            continue;
-          }
-          // this cell is the low side ('a') of its high face, 'b' of its low face
-          accE += (sd ? a.jc[slot] : a.jc[NS + slot]) * lE;
-          accT += a.jc[2 * NS + slot] * lE + (sd ? a.jc[3 * NS + slot] : a.jc[4 * NS + slot]) * lT;
-          accZ += a.jc[5 * NS + slot] * lE;
-        }
+      const int g = P.goff + P.fo[f] + pos[(d + 1) % 3] + P.n[(d + 1) % 3] * pos[(d + 2) % 3];
+      const uint8_t ty = a.gtype[g];
+      if (ty == GT_NEUMANN) continue;
+      const double* jf = J.jc + 3L * N + g;
+      if (DZ) aZ = fma(jf[5 * NS], face_adj(a, wE, idx, g, hi, ty), aZ);
+      if (ty == GT_CF) {
+        // the coarse cell's share of this face (the cell's own is in cen)
+        const int C = a.gzsrc[g];
+        const double lE = (hi ? -0.125 : 0.125) * wE[C], lT = (hi ? -0.125 : 0.125) * wT[C];
+        aE = fma(hi ? jf[0] : jf[NS], lE, aE);
+        aT = fma(jf[2 * NS], lE, aT);
+        aT = fma(hi ? jf[3 * NS] : jf[4 * NS], lT, aT);
       }
-      // ghosts that read this cell (sibling copies, coarse-fine stencils)
-      for (int q = a.ts_off[idx]; q < a.ts_off[idx + 1]; q++) {
-        const int g = a.ts_g[q];
-        const double wq = a.ts_w[q];
-        accE += wq * a.gam[g];
-        accT += wq * a.gam[G + g];
-      }
-      const double wE = a.w[idx], wT = a.w[N + idx];
-      const double dw = wE - wT;
-      a.out[idx] = a.a0 * wE - a.dt * (accE + a.cc[idx] * dw);
-      a.out[N + idx] = a.a0 * wT - a.dt * (accT + a.cc[N + idx] * dw);
-      if (a.dz) {
-        for (int q = a.tz_off[idx]; q < a.tz_off[idx + 1]; q++) accZ += a.gam[2L * G + a.tz_g[q]];
-        const double zc = (double)a.z[idx];
-        a.dz[idx] = -a.dt * 3.0 * zc * zc * (accZ + a.cc[2L * N + idx] * dw);
-      }
+    }
+    // ghosts that read this cell (sibling copies, coarse-fine stencils)
+    for (int t = a.ts_off[idx]; t < a.ts_off[idx + 1]; t++) {
+      const int g = a.ts_g[t];
+      const double wq = a.ts_w[t];
+      aE += wq * a.gam[g];
+      aT += wq * a.gam[G + g];
+    }
+    a.out[idx] = fma(-a.dt, aE, soft_mul_any(a.a0, wEc));
+    a.out[N + idx] = fma(-a.dt, aT, soft_mul_any(a.a0, wTc));
+    if (DZ) {
+      for (int t = a.tz_off[idx]; t < a.tz_off[idx + 1]; t++) aZ += a.gam[2 * G + a.tz_g[t]];
+      const double zc = (double)a.z[idx];
+      a.dz[idx] = -a.dt * 3.0 * zc * zc * (aZ + J.cZ[idx] * (wEc - wTc));
     }
   }
 }
 
 }  // namespace
 
-void launch_vjp(const Hier& H, const double* jc, const double* cc, const float* z, const double* w,
-                double* lam, double* gam, double a0, double dt, double* out, double* dz,
-                cudaStream_t s) {
+void launch_vjp(const Hier& H, const Jac& jac, const float* z, const double* w, double* gam,
+                double a0, double dt, double* out, double* dz, cudaStream_t s) {
   VjpArgs a;
   a.tiles = H.d_tiles;
   a.patches = H.d_patches;
@@ -223,11 +173,9 @@ void launch_vjp(const Hier& H, const double* jc, const double* cc, const float* 
   a.ts_w = H.d_ts_w;
   a.tz_off = H.d_tz_off;
   a.tz_g = H.d_tz_g;
-  a.jc = jc;
-  a.cc = cc;
+  a.jac = jac;
   a.z = z;
   a.w = w;
-  a.lam = lam;
   a.gam = gam;
   a.out = out;
   a.dz = dz;
@@ -235,13 +183,12 @@ void launch_vjp(const Hier& H, const double* jc, const double* cc, const float* 
   a.dt = dt;
   a.N = H.N;
   a.G = H.G;
-  a.ntiles = (int)H.tiles.size();
   a.tx = H.tile_x;
   a.ty = H.tile_y;
-  a.tz = H.tile_z;
   const int nt = std::max(1, (int)H.tiles.size());
-  k_vjp_faces<<<nt, 256, 0, s>>>(a);
+  const int bs = std::min(256, H.tile_x * H.tile_y * H.tile_z);
   int gb = (int)std::min(152L * 8, (H.G + 255L) / 256);
   k_vjp_ghosts<<<std::max(gb, 1), 256, 0, s>>>(a);
-  k_vjp_cells<<<nt, 256, 0, s>>>(a);
+  if (dz) k_vjp_cells<true><<<nt, bs, 0, s>>>(a);
+  else k_vjp_cells<false><<<nt, bs, 0, s>>>(a);
 }

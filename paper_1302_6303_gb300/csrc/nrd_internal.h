@@ -123,14 +123,30 @@ int hier_tiles(Hier& H, std::string& err);
 void hier_free(Hier& H);
 
 // Kernel launchers (k_stencil.cu)
-// stencil modes; ST_JVF applies the Jacobian frozen by ST_LIN (jc, cc) to v;
+// stencil modes (the frozen Jv has a kernel of its own, launch_jv_frozen);
 // ST_LINZ is ST_LIN that also forms the partials with respect to z^3.
 // The residual and the linearisation run as two launches (ST_RESF / ST_RESC,
 // ST_LINF / ST_LINC, ST_LINZF / ST_LINZC): every face once, its flux over h to
 // StencilIO::pef, then the cell balance from them.  Every face flux and flux
 // partial is kept divided by h (its share of a cell's divergence).
-enum { ST_RESIDUAL = 0, ST_JV = 1, ST_FD = 2, ST_LIN = 3, ST_JVF = 4, ST_LINZ = 5, ST_LINF = 6,
+enum { ST_RESIDUAL = 0, ST_JV = 1, ST_FD = 2, ST_LIN = 3, ST_LINZ = 5, ST_LINF = 6,
        ST_LINC = 7, ST_RESF = 8, ST_RESC = 9, ST_LINZF = 10, ST_LINZC = 11 };
+// The Jacobian frozen by the linearisation, L = f' (the residual's tangent is
+// a0 v - dt L v): the partials of every face flux over h (face slots [3N low
+// faces | G patch-boundary faces]; a is the face's low side, b its high one) and,
+// per cell, its own entries in its two rows: the sums of its faces' partials
+// and of the coupling.  A product is then one sum per row.  Faces taken by
+// flux matching (cell mask bits) are not in the own entries.
+//   jc[q (3N + G) + slot]   d Phi_E / d E_a, E_b, T (a or b); d Phi_T / d T_a, T_b;
+//                           d Phi_E / d z^3 (a or b)
+//   cen[q N + c]            EE, ET, TT, TE
+//   cZ[c]                   d coupling / d z^3
+// (Robin faces: slots 0 and 1 both d Phi_E / d E_c, slot 2 d Phi_E / d T_c.)
+struct Jac {
+  double* jc = nullptr;   // [6][3N + G]
+  double* cen = nullptr;  // [4][N]
+  double* cZ = nullptr;   // [N]
+};
 struct StencilIO {
   const double* u;      // state (E then T)
   const double* v;      // direction (JV, FD)
@@ -143,9 +159,8 @@ struct StencilIO {
   double* out;          // F or Jv
   double* cfflux;       // [2][G] fine-side coarse-fine fluxes
   // ST_LIN outputs (face slots: [3N low faces | G boundary faces])
-  double* jc;           // [6][3N+G] flux partial derivatives (5: d Phi_E / d z^3)
+  Jac jac;              // frozen Jacobian (also read by the frozen Jv)
   double* craw;         // [2][3N+G] frozen D_E, D_T (Robin slots: D_b)
-  double* cc;           // [3][N] coupling partials (E, T, z^3)
   double beta;          // dt / a0
   float* a32;           // [2][3N+G] scaled P1 coefficients (FP32 V-cycle), or
   double* a64;          //   the FP64 array when a32 is null
@@ -157,18 +172,17 @@ struct StencilIO {
 void launch_ghost_fill(const Hier& H, const ModelParams& mp, const float* z, const double* u,
                        double* g, int nonlinear, cudaStream_t s);
 void launch_ghost_z(const Hier& H, const float* z, float* gz, cudaStream_t s);
-// z3: z^3 in FP64 for the cells followed by the ghosts (N + G); not read by ST_JVF
+// z3: z^3 in FP64 for the cells followed by the ghosts (N + G)
 void launch_stencil(const Hier& H, const ModelParams& mp, int mode, const StencilIO& io,
                     cudaStream_t s, const double* z3);
 // z3[c] = z[c]^3 (cells), z3[N + g] = gz[g]^3 (ghosts), in FP64
 void launch_cube(const Hier& H, const float* z, const float* gz, double* z3, cudaStream_t s);
 void launch_reflux(const Hier& H, const StencilIO& io, int mode, cudaStream_t s);
-void launch_jv_frozen(const Hier& H, const ModelParams& mp, const double* jc, const double* cc,
-                      const StencilIO& io, cudaStream_t s);
+// Jv = a0 v - dt L v with the frozen Jacobian io.jac
+void launch_jv_frozen(const Hier& H, const StencilIO& io, cudaStream_t s);
 // k_vjp.cu: JTw = (dF/du)^T w, dz = (dF/dz)^T w (dz may be null)
-void launch_vjp(const Hier& H, const double* jc, const double* cc, const float* z, const double* w,
-                double* lam, double* gam, double a0, double dt, double* out, double* dz,
-                cudaStream_t s);
+void launch_vjp(const Hier& H, const Jac& jac, const float* z, const double* w, double* gam,
+                double a0, double dt, double* out, double* dz, cudaStream_t s);
 void launch_tag(const Hier& H, const double* E, const double* gE, double thr_c, double thr_g,
                 double thr_r, const double* emax, uint8_t* tags, cudaStream_t s);
 void launch_average_down(const Hier& H, double* x, int nfield, int fstride, cudaStream_t s);
@@ -316,10 +330,8 @@ struct nrd_ctx {
   double* d_gv = nullptr;      // 2G: ghosts of a direction
   double* d_cf = nullptr;      // 2G: fine-side coarse-fine fluxes
   double* d_tmp = nullptr;     // 2N scratch
-  double* d_jc = nullptr;      // [6][3N+G] frozen flux partial derivatives
+  Jac jac;                     // frozen Jacobian (one allocation, at jac.jc)
   double* d_pef = nullptr;     // [2][3N+G] face fluxes of the split linearisation
-  double* d_cc = nullptr;      // [3][N] frozen coupling partials
-  double* d_lam = nullptr;     // [2][3N+G] adjoint face scratch
   double* d_gam = nullptr;     // [3][G] adjoint ghost scratch
   double* d_z3 = nullptr;      // [N + G] z^3 of cells and ghost cells (FP64)
   bool lin_ready = false;

@@ -80,6 +80,18 @@ __device__ __forceinline__ double soft_twice(double x) {
   return __hiloint2double((int)((h << 1) ? h + 0x100000u : h), (int)dbl_lo(x));
 }
 
+// x y for any x, y: on the integer pipe where both lie within 2^(+-480) (the
+// product is then normal), else one native multiplication behind a call (a
+// predicated one would take its FP64 slot in every warp)
+static __device__ __noinline__ double native_mul(double x, double y) { return __dmul_rn(x, y); }
+__device__ __forceinline__ double soft_mul_any(double x, double y) {
+  const unsigned xm = dbl_hi(x) & 0x7fffffffu, ym = dbl_hi(y) & 0x7fffffffu;
+  constexpr unsigned lo = (1023u - 480u) << 20, w = 960u << 20;
+  if (xm - lo >= w || ym - lo >= w) return native_mul(x, y);
+  return __longlong_as_double((long long)(soft_mul_bits(x, y) |
+      ((uint64_t)((dbl_hi(x) ^ dbl_hi(y)) & 0x80000000u) << 32)));
+}
+
 // the products of a face's or a cell's formulas, on the integer pipe (SOFT)
 // or native; the same bits either way
 template <bool SOFT>

@@ -209,7 +209,7 @@ static int gmres(nrd_ctx* c, const double* u, const double* b, double a0, double
   const int mode = (c->p.jv_mode == NRD_JV_ANALYTIC) ? NRD_JV_FROZEN : NRD_JV_FD;
   auto apply = [&](const double* v, double* out) -> int {
     if (transposed) {
-      launch_vjp(H, c->d_jc, c->d_cc, c->d_z, v, c->d_lam, c->d_gam, a0, dt, out, nullptr, s);
+      launch_vjp(H, c->jac, c->d_z, v, c->d_gam, a0, dt, out, nullptr, s);
       return cudaGetLastError() == cudaSuccess ? NRD_OK : NRD_ECUDA;
     }
     return ctx_jv(c, u, v, b, c->d_F, a0, dt, mode, out, false, s);
@@ -408,7 +408,7 @@ int solver_adjoint(nrd_ctx* c, const double* g, double a0, double dt, double rto
   if (rc != NRD_OK) return rc;
   cudaMemcpyAsync(lam, c->d_dx, n2 * sizeof(double), cudaMemcpyDeviceToDevice, s);
   // final residual of the adjoint system
-  launch_vjp(H, c->d_jc, c->d_cc, c->d_z, lam, c->d_lam, c->d_gam, a0, dt, c->d_w, nullptr, s);
+  launch_vjp(H, c->jac, c->d_z, lam, c->d_gam, a0, dt, c->d_w, nullptr, s);
   k_resid<<<grid1(n2), 256, 0, s>>>(n2, g, 1.0, c->d_w, c->d_r);
   launch_wdot_lv(H, c->R, c->d_r, c->d_r, SL_R, s);
   double rn = std::sqrt(read_slot(c, SL_R, s));

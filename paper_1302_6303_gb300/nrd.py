@@ -200,8 +200,9 @@ def check_narrow(x):
 
 
 def check_softmul(x, y):
-    """[integer-pipe x y, __dmul_rn(x, y), integer-pipe 2 x] (nrd_check_softmul)."""
-    out = torch.empty(3, x.numel(), dtype=torch.float64, device=x.device)
+    """[integer-pipe x y, __dmul_rn(x, y), integer-pipe 2 x, x y with a native
+    fallback] (nrd_check_softmul)."""
+    out = torch.empty(4, x.numel(), dtype=torch.float64, device=x.device)
     rc = load().nrd_check_softmul(_ptr(x, torch.float64), _ptr(y, torch.float64), x.numel(),
                                   _ptr(out, torch.float64), _stream())
     if rc != OK:

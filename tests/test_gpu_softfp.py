@@ -59,6 +59,11 @@ def test_product_bits(nrd):
     got = nrd.check_softmul(dev(x), dev(y)).cpu().numpy()
     np.testing.assert_array_equal(got[0].view(np.uint64), got[1].view(np.uint64))
     np.testing.assert_array_equal(got[0].view(np.uint64), (x * y).view(np.uint64))
+    # with the fallback: every operand, the ends of the range and nan included
+    ends = np.array([5e-324, -3e-310, 1e-308, 1e308, -1e308, np.inf, -np.inf, np.nan, 0.0, 1.5])
+    c, d = (q.ravel() for q in np.meshgrid(ends, ends))
+    any_ = nrd.check_softmul(dev(np.concatenate([x, c])), dev(np.concatenate([y, d])))
+    np.testing.assert_array_equal(any_[3].cpu().numpy(), any_[1].cpu().numpy())
     low = np.abs(x) < 2.0 ** 1000
     np.testing.assert_array_equal(got[2][low].view(np.uint64), (2 * x[low]).view(np.uint64))
 
