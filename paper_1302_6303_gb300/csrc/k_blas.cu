@@ -462,19 +462,6 @@ __device__ void grid_barrier(unsigned* bar, int* err) {
   __syncthreads();
 }
 
-// every block sums the nq block partials (stride NVMAX) in block order into
-// out[0..nq) (shared); the same order in every block, so all agree
-__device__ void coop_reduce(const double* part, int nq, double* out, double* sh) {
-  for (int q = 0; q < nq; q++) {
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
-      acc += __ldcg(&part[(long)b * NVMAX + q]);
-    const double r = block_red<0>(acc, sh);
-    if (threadIdx.x == 0) out[q] = r;
-    __syncthreads();
-  }
-}
-
 // Volume weights of a level-major vector whose covered cells are zero (every
 // Krylov vector, F and the Newton directions): the leaf-cell volume is
 // constant on a level, so a weighted dot is, per level, an FMA chain over
@@ -486,110 +473,187 @@ struct LevW {
   double w[NRD_MAX_LEVELS];    // cell volume of level l
 };
 
-// One sweep over a thread's cells (level-weighted, see LevW): with UPD first
-// w -= sum_{q<nv} hu_q V_q (stored back), then the NQ dots
-// <w, V_{q0+q}> and, with NORM, <w, w>.  NQ, UPD and NORM are compile-time,
-// so no FP64 instruction is issued for an unused accumulator.  Block
-// partials to part[blockIdx.x * NVMAX + col0 + q] (the norm after the dots).
-template <int NQ, bool UPD, bool NORM>
-__device__ void orth_sweep(const LevW& lw, int l0, double* __restrict__ w,
-                           const double* __restrict__ V, long stride, int N, int nv,
-                           const double* hu, int q0, double* part, int col0, double* sh) {
-  constexpr int NA = NQ + (NORM ? 1 : 0);
-  double acc[NA > 0 ? NA : 1], tot[NA > 0 ? NA : 1];
+// Columns handled by one sweep: their loads are all in flight together.
+constexpr int OQ = 8;
+
+// The NA accumulators of every thread summed over the block: warp w takes
+// quantity w, w + 8, ... (each lane 8 threads' values, then the warp's tree), so
+// all of them cost one pass of 12 FP64 warp additions and one barrier; a block
+// tree per quantity cost nine barriers each.  Quantity q goes to
+// part[col_q * gridDim.x + blockIdx.x] (col_q = col0 + q, the last one to colN
+// when NORM).  sh: at least NA * 256 doubles; 256 threads.
+template <int NA, bool NORM>
+__device__ __forceinline__ void block_parts(const double (&acc)[NA], double* part, int col0,
+                                            int colN, double* sh) {
+  const int t = threadIdx.x, lane = t & 31;
+  __syncthreads();   // sh may still be read by a previous call
 #pragma unroll
-  for (int q = 0; q < NA; q++) acc[q] = tot[q] = 0.0;
-  const int T = gridDim.x * blockDim.x;
-  int l = l0, lend = lw.end[l0];
-  double lwt = lw.w[l0];
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += T) {
-    while (i >= lend) {
-#pragma unroll
-      for (int q = 0; q < NA; q++) {
-        tot[q] = fma(lwt, acc[q], tot[q]);
-        acc[q] = 0.0;
-      }
-      l++;
-      lend = lw.end[l];
-      lwt = lw.w[l];
-    }
-    double wE = w[i], wT = w[N + i];
-    if (UPD) {
-      for (int q = 0; q < nv; q++) {
-        wE = fma(-hu[q], V[q * stride + i], wE);
-        wT = fma(-hu[q], V[q * stride + N + i], wT);
-      }
-      w[i] = wE;
-      w[N + i] = wT;
-    }
-#pragma unroll
-    for (int q = 0; q < NQ; q++)
-      acc[q] = fma(wE, V[(q0 + q) * stride + i], fma(wT, V[(q0 + q) * stride + N + i], acc[q]));
-    if (NORM) acc[NA - 1] = fma(wE, wE, fma(wT, wT, acc[NA - 1]));
-  }
-#pragma unroll
-  for (int q = 0; q < NA; q++) {
-    tot[q] = fma(lwt, acc[q], tot[q]);
-    const double r = block_red<0>(tot[q], sh);
-    if (threadIdx.x == 0) part[(long)blockIdx.x * NVMAX + col0 + q] = r;
+  for (int q = 0; q < NA; q++) sh[q * RB + t] = acc[q];
+  __syncthreads();
+  for (int q = t >> 5; q < NA; q += RB / 32) {
+    const double* v = sh + q * RB + lane;
+    double r = ((v[0] + v[32]) + (v[64] + v[96])) + ((v[128] + v[160]) + (v[192] + v[224]));
+    r = warp_sum(r);
+    const int col = (NORM && q == NA - 1) ? colN : col0 + q;
+    if (lane == 0) part[(long)col * gridDim.x + blockIdx.x] = r;
   }
 }
 
-// the dots <w, V_q>, q < nv, in chunks of 4 (UPD and NORM on the first chunk)
-template <bool UPD, bool NORM>
-__device__ void orth_dots(const LevW& lw, int l0, double* w, const double* V, long stride, int N,
-                          int nv, const double* hu, double* part, double* sh) {
-  for (int q0 = 0; q0 < nv; q0 += 4) {
-    const int nq = min(4, nv - q0);
-    const bool first = (q0 == 0);
-    // norm column: right after the last dot (col nv)
-    if (first) {
-      switch (nq) {
-        case 1: orth_sweep<1, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, 0, sh); break;
-        case 2: orth_sweep<2, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, 0, sh); break;
-        case 3: orth_sweep<3, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, 0, sh); break;
-        default: orth_sweep<4, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, 0, sh);
-      }
-      if (NORM && nq < nv && threadIdx.x == 0) {
-        // move the norm partial from column nq to column nv
-        part[(long)blockIdx.x * NVMAX + nv] = part[(long)blockIdx.x * NVMAX + nq];
-      }
-    } else {
-      switch (nq) {
-        case 1: orth_sweep<1, false, false>(lw, l0, w, V, stride, N, nv, hu, q0, part, q0, sh); break;
-        case 2: orth_sweep<2, false, false>(lw, l0, w, V, stride, N, nv, hu, q0, part, q0, sh); break;
-        case 3: orth_sweep<3, false, false>(lw, l0, w, V, stride, N, nv, hu, q0, part, q0, sh); break;
-        default: orth_sweep<4, false, false>(lw, l0, w, V, stride, N, nv, hu, q0, part, q0, sh);
-      }
+// sums of the block partials of nq quantities in a fixed order (the same in
+// every block) -> out (shared): one quantity per warp at a time
+__device__ void coop_sum(const double* part, int nq, double* out) {
+  const int lane = threadIdx.x & 31, nb = gridDim.x;
+  for (int q = threadIdx.x >> 5; q < nq; q += blockDim.x >> 5) {
+    const double* v = part + (long)q * nb;
+    double a0 = 0.0, a1 = 0.0;
+    int b = lane;
+    for (; b + 32 < nb; b += 64) {
+      a0 += __ldcg(v + b);
+      a1 += __ldcg(v + b + 32);
     }
-  }
-}
-
-// sums of block partials in block order (the same in every block) -> out
-__device__ void coop_sum(const double* part, int nq, double* out, double* sh) {
-  for (int q = 0; q < nq; q++) {
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
-      acc += __ldcg(&part[(long)b * NVMAX + q]);
-    const double r = block_red<0>(acc, sh);
-    if (threadIdx.x == 0) out[q] = r;
+    if (b < nb) a0 += __ldcg(v + b);
+    const double r = warp_sum(a0 + a1);
+    if (lane == 0) out[q] = r;
   }
   __syncthreads();
 }
 
-// V[nv] = (w - V h) * sc, one sweep
-__device__ void orth_final(double* __restrict__ w, double* __restrict__ V, long stride, int N,
-                           int nv, const double* h, double sc) {
+// (wE, wT) -= sum_{q < NQ} h_q V_q at cell i
+template <int NQ>
+__device__ __forceinline__ void sub_cols(double& wE, double& wT, const double* __restrict__ V,
+                                         long stride, long i, long N, const double* h) {
+  double a[NQ], b[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; q++) {
+    a[q] = V[q * stride + i];
+    b[q] = V[q * stride + N + i];
+  }
+#pragma unroll
+  for (int q = 0; q < NQ; q++) {
+    wE = fma(-h[q], a[q], wE);
+    wT = fma(-h[q], b[q], wT);
+  }
+}
+// the same over nv columns: OQ at a time, the rest one by one
+__device__ __forceinline__ void sub_all(double& wE, double& wT, const double* __restrict__ V,
+                                        long stride, long i, long N, int nv, const double* h) {
+  int q = 0;
+  for (; q + OQ <= nv; q += OQ) sub_cols<OQ>(wE, wT, V + q * stride, stride, i, N, h + q);
+  for (; q < nv; q++) sub_cols<1>(wE, wT, V + q * stride, stride, i, N, h + q);
+}
+
+// One sweep over a thread's cells (level-weighted, see LevW; a level's cells
+// have 1/8 of the volume of the coarser level's, so the sum so far times 8
+// carries over exactly): with UPD first w -= sum_{q<nv} hu_q V_q (stored
+// back), then the NQ dots <w, V_{q0+q}> and, with NORM, <w, w>.  NQ, UPD and
+// NORM are compile-time, so no FP64 instruction is issued for an unused
+// accumulator, and the loads of a cell are in flight together.
+template <int NQ, bool UPD, bool NORM>
+__device__ __forceinline__ void orth_sweep(const LevW& lw, int l0, double* __restrict__ w,
+                                        const double* __restrict__ V, long stride, int N, int nv,
+                                        const double* hu, int q0, double* part, double* sh) {
+  constexpr int NA = NQ + (NORM ? 1 : 0);
+  double acc[NA];
+#pragma unroll
+  for (int q = 0; q < NA; q++) acc[q] = 0.0;
+  const int T = gridDim.x * blockDim.x;
+  int l = l0, lend = lw.end[l0];
+  const double* Vq = V + q0 * stride;
+#pragma unroll(NQ <= 2 ? 2 : 1)
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += T) {
+    while (i >= lend) {
+#pragma unroll
+      for (int q = 0; q < NA; q++) acc[q] *= 8.0;
+      lend = lw.end[++l];
+    }
+    double wE = w[i], wT = w[N + i];
+    double a[NQ], b[NQ];
+    if (UPD && NQ < OQ) {
+      // all nv = NQ columns: loaded once for the update and the dots
+#pragma unroll
+      for (int q = 0; q < NQ; q++) {
+        a[q] = Vq[q * stride + i];
+        b[q] = Vq[q * stride + N + i];
+      }
+#pragma unroll
+      for (int q = 0; q < NQ; q++) {
+        wE = fma(-hu[q], a[q], wE);
+        wT = fma(-hu[q], b[q], wT);
+      }
+    } else {
+      if (UPD) sub_all(wE, wT, V, stride, i, N, nv, hu);
+#pragma unroll
+      for (int q = 0; q < NQ; q++) {
+        a[q] = Vq[q * stride + i];
+        b[q] = Vq[q * stride + N + i];
+      }
+    }
+    if (UPD) {
+      w[i] = wE;
+      w[N + i] = wT;
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; q++) acc[q] = fma(wE, a[q], fma(wT, b[q], acc[q]));
+    if (NORM) acc[NA - 1] = fma(wE, wE, fma(wT, wT, acc[NA - 1]));
+  }
+#pragma unroll
+  for (int q = 0; q < NA; q++) acc[q] *= lw.w[l];
+  block_parts<NA, NORM>(acc, part, q0, nv, sh);
+}
+
+// the dots <w, V_q>, q < nv, in sweeps of up to OQ (UPD and NORM on the first)
+template <bool UPD, bool NORM>
+__device__ __forceinline__ void orth_dots(const LevW& lw, int l0, double* w, const double* V, long stride, int N,
+                          int nv, const double* hu, double* part, double* sh) {
+  const int n = min(OQ, nv);
+  switch (n) {
+    case 1: orth_sweep<1, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, sh); break;
+    case 2: orth_sweep<2, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, sh); break;
+    case 3: orth_sweep<3, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, sh); break;
+    case 4: orth_sweep<4, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, sh); break;
+    case 5: orth_sweep<5, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, sh); break;
+    case 6: orth_sweep<6, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, sh); break;
+    case 7: orth_sweep<7, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, sh); break;
+    default: orth_sweep<8, UPD, NORM>(lw, l0, w, V, stride, N, nv, hu, 0, part, sh);
+  }
+  int q0 = OQ;
+  for (; q0 + OQ <= nv; q0 += OQ)
+    orth_sweep<8, false, false>(lw, l0, w, V, stride, N, nv, hu, q0, part, sh);
+  for (; q0 + 4 <= nv; q0 += 4)
+    orth_sweep<4, false, false>(lw, l0, w, V, stride, N, nv, hu, q0, part, sh);
+  switch (nv - q0) {
+    case 1: orth_sweep<1, false, false>(lw, l0, w, V, stride, N, nv, hu, q0, part, sh); break;
+    case 2: orth_sweep<2, false, false>(lw, l0, w, V, stride, N, nv, hu, q0, part, sh); break;
+    case 3: orth_sweep<3, false, false>(lw, l0, w, V, stride, N, nv, hu, q0, part, sh); break;
+    default: break;
+  }
+}
+
+// V[nv] = (w - V h) * sc, one sweep; NV > 0: all nv = NV columns at once
+template <int NV>
+__device__ __forceinline__ void orth_final_n(const double* __restrict__ w, double* __restrict__ V,
+                                             long stride, int N, int nv, const double* h,
+                                             double sc) {
   const int T = gridDim.x * blockDim.x;
   double* vn = V + (long)nv * stride;
+#pragma unroll(NV == 1 || NV == 2 ? 2 : 1)
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += T) {
     double wE = w[i], wT = w[N + i];
-    for (int q = 0; q < nv; q++) {
-      wE = fma(-h[q], V[q * stride + i], wE);
-      wT = fma(-h[q], V[q * stride + N + i], wT);
-    }
+    if (NV > 0) sub_cols<(NV > 0 ? NV : 1)>(wE, wT, V, stride, i, N, h);
+    else sub_all(wE, wT, V, stride, i, N, nv, h);
     vn[i] = sc * wE;
     vn[N + i] = sc * wT;
+  }
+}
+__device__ __forceinline__ void orth_final(const double* w, double* V, long stride, int N, int nv,
+                           const double* h, double sc) {
+  switch (nv) {
+    case 1: orth_final_n<1>(w, V, stride, N, nv, h, sc); break;
+    case 2: orth_final_n<2>(w, V, stride, N, nv, h, sc); break;
+    case 3: orth_final_n<3>(w, V, stride, N, nv, h, sc); break;
+    case 4: orth_final_n<4>(w, V, stride, N, nv, h, sc); break;
+    case 5: orth_final_n<5>(w, V, stride, N, nv, h, sc); break;
+    default: orth_final_n<0>(w, V, stride, N, nv, h, sc);
   }
 }
 
@@ -615,15 +679,19 @@ constexpr double kReorthFrac = 1e-4;
 // res[slot_nrm] = the squared norm of the orthogonalised w.  Partials
 // ping-pong between pa and pb so that each reduction needs one barrier.
 // Every block sums the partials in the same order, so all take the same
-// branch.  always2: the second pass every time (CGS2; solves that need an
+// branch.  Bound by latency on small vectors (loads, the reduction trees and
+// the grid barrier) and by the FP64 pipe and HBM together on large ones.  Per
+// call of a step's solves, against block trees per quantity and columns loaded
+// one after the other: 32^3 21.6 -> 12.9 us, base 64^3 + fine band (0.5M cells)
+// 52.3 -> 42.1 us, 256^3 647 -> 570 us.  always2: the second pass every time (CGS2; solves that need an
 // orthogonal basis to working precision, such as the adjoint's).
-__global__ void __launch_bounds__(256) k_orth_coop(LevW lw, double* __restrict__ w,
+__global__ void __launch_bounds__(RB, 3) k_orth_coop(LevW lw, double* __restrict__ w,
                                                    double* __restrict__ V, long stride, int N,
                                                    const int* jd, int add, double* pa, double* pb,
                                                    unsigned* bar, int* err, double* res,
                                                    int slot_h1, int slot_h2, int slot_nrm,
                                                    int always2) {
-  __shared__ double sh[1024];
+  __shared__ double sh[(OQ + 1) * RB];
   __shared__ double h[NVMAX + 1];
   __shared__ double hu[NVMAX];
   __shared__ double s_sc, s_nrm;
@@ -635,7 +703,7 @@ __global__ void __launch_bounds__(256) k_orth_coop(LevW lw, double* __restrict__
 
   orth_dots<false, true>(lw, l0, w, V, stride, N, nv, nullptr, pa, sh);
   grid_barrier(bar, err);
-  coop_sum(pa, nv + 1, h, sh);                   // h = h1, h[nv] = |w|^2
+  coop_sum(pa, nv + 1, h);                   // h = h1, h[nv] = |w|^2
   if (threadIdx.x == 0) {
     double q2 = 0.0;
     for (int q = 0; q < nv; q++) q2 = fma(h[q], h[q], q2);
@@ -658,7 +726,7 @@ __global__ void __launch_bounds__(256) k_orth_coop(LevW lw, double* __restrict__
   }
   orth_dots<true, true>(lw, l0, w, V, stride, N, nv, hu, pb, sh);
   grid_barrier(bar, err);
-  coop_sum(pb, nv + 1, h, sh);                   // h = h2, h[nv] = |w|^2
+  coop_sum(pb, nv + 1, h);                   // h = h2, h[nv] = |w|^2
   if (threadIdx.x == 0) {
     double q2 = 0.0;
     for (int q = 0; q < nv; q++) q2 = fma(h[q], h[q], q2);
@@ -711,28 +779,30 @@ int grid_for(long n) {
 
 int reducer_init(Reducer& R, int N) {
   R.nblk = std::max(1, std::min((N + RB * 4 - 1) / (RB * 4), 152 * 4));
-  if (cudaMalloc(&R.d_part, sizeof(double) * (size_t)R.nblk * NVMAX) != cudaSuccess) return NRD_ENOMEM;
-  if (cudaMalloc(&R.d_res, sizeof(double) * 256) != cudaSuccess) return NRD_ENOMEM;
-  if (cudaMallocHost(&R.h_res, sizeof(double) * 256) != cudaSuccess) return NRD_ENOMEM;
-  if (cudaMalloc(&R.d_count, sizeof(unsigned)) != cudaSuccess) return NRD_ENOMEM;
-  if (cudaMalloc(&R.d_bar, 2 * sizeof(unsigned)) != cudaSuccess) return NRD_ENOMEM;
-  if (cudaMalloc(&R.d_part2, sizeof(double) * (size_t)R.nblk * NVMAX) != cudaSuccess)
-    return NRD_ENOMEM;
-  if (cudaMalloc(&R.d_err, sizeof(int)) != cudaSuccess) return NRD_ENOMEM;
-  cudaMemset(R.d_res, 0, sizeof(double) * 256);
-  cudaMemset(R.d_count, 0, sizeof(unsigned));
-  cudaMemset(R.d_bar, 0, 2 * sizeof(unsigned));
-  cudaMemset(R.d_err, 0, sizeof(int));
-  // cooperative CGS2: every block resident, at most the partial buffer's rows
+  // cooperative Gram-Schmidt: every block resident; one block per 256 cells up
+  // to a full machine (small vectors want every load in flight at once more
+  // than few partials)
   {
     int dev = 0, nsm = 0, per = 0, coop = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_orth_coop, RB, 0);
-    int want = std::max(1, (N + RB - 1) / RB);
-    R.coop_blocks = coop ? std::min(std::min(nsm * std::min(per, 4), want), R.nblk) : 0;
+    const int want = std::max(1, (N + RB - 1) / RB);
+    R.coop_blocks = coop ? std::min(nsm * std::min(per, 4), want) : 0;
   }
+  const size_t np = (size_t)std::max(R.nblk, R.coop_blocks) * NVMAX;
+  if (cudaMalloc(&R.d_part, sizeof(double) * np) != cudaSuccess) return NRD_ENOMEM;
+  if (cudaMalloc(&R.d_res, sizeof(double) * 256) != cudaSuccess) return NRD_ENOMEM;
+  if (cudaMallocHost(&R.h_res, sizeof(double) * 256) != cudaSuccess) return NRD_ENOMEM;
+  if (cudaMalloc(&R.d_count, sizeof(unsigned)) != cudaSuccess) return NRD_ENOMEM;
+  if (cudaMalloc(&R.d_bar, 2 * sizeof(unsigned)) != cudaSuccess) return NRD_ENOMEM;
+  if (cudaMalloc(&R.d_part2, sizeof(double) * np) != cudaSuccess) return NRD_ENOMEM;
+  if (cudaMalloc(&R.d_err, sizeof(int)) != cudaSuccess) return NRD_ENOMEM;
+  cudaMemset(R.d_res, 0, sizeof(double) * 256);
+  cudaMemset(R.d_count, 0, sizeof(unsigned));
+  cudaMemset(R.d_bar, 0, 2 * sizeof(unsigned));
+  cudaMemset(R.d_err, 0, sizeof(int));
   return NRD_OK;
 }
 
