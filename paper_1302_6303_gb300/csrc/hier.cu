@@ -545,7 +545,6 @@ int hier_upload(Hier& H, std::string& err) {
   UP(H.d_rf_off, rf_off);
   UP(H.d_rf_face, rf_face);
   UP(H.d_rf_g, rf_g);
-  UP(H.d_rf_level, rf_level);
   UP(H.d_ts_off, ts_off);
   UP(H.d_ts_g, ts_g);
   UP(H.d_ts_w, ts_w);
@@ -634,7 +633,7 @@ void hier_free(Hier& H) {
   };
   F(H.d_patches); F(H.d_tiles); F(H.d_mask); F(H.d_wvol); F(H.d_gtype); F(H.d_gface);
   F(H.d_gcell); F(H.d_gzsrc); F(H.d_gt0); F(H.d_gidx); F(H.d_gw); F(H.d_rf_cell);
-  F(H.d_rf_off); F(H.d_rf_face); F(H.d_rf_g); F(H.d_rf_level);
+  F(H.d_rf_off); F(H.d_rf_face); F(H.d_rf_g);
   F(H.d_ts_off); F(H.d_ts_g); F(H.d_ts_w); F(H.d_tz_off); F(H.d_tz_g);
   H.d_ts_off = nullptr; H.d_ts_g = nullptr; H.d_ts_w = nullptr; H.d_tz_off = nullptr;
   H.d_tz_g = nullptr;
@@ -646,5 +645,5 @@ void hier_free(Hier& H) {
   H.d_patches = nullptr; H.d_tiles = nullptr; H.d_mask = nullptr; H.d_wvol = nullptr;
   H.d_gtype = nullptr; H.d_gface = nullptr; H.d_gcell = nullptr; H.d_gzsrc = nullptr;
   H.d_gt0 = nullptr; H.d_gidx = nullptr; H.d_gw = nullptr; H.d_rf_cell = nullptr;
-  H.d_rf_off = nullptr; H.d_rf_face = nullptr; H.d_rf_g = nullptr; H.d_rf_level = nullptr;
+  H.d_rf_off = nullptr; H.d_rf_face = nullptr; H.d_rf_g = nullptr;
 }

@@ -684,13 +684,15 @@ constexpr double kReorthFrac = 1e-4;
 // call of a step's solves, against block trees per quantity and columns loaded
 // one after the other: 32^3 21.6 -> 12.9 us, base 64^3 + fine band (0.5M cells)
 // 52.3 -> 42.1 us, 256^3 647 -> 570 us.  always2: the second pass every time (CGS2; solves that need an
-// orthogonal basis to working precision, such as the adjoint's).
+// orthogonal basis to working precision, such as the adjoint's).  end (end.c
+// non-null): block 0 ends the Arnoldi step of the Newton graph while the others
+// form V[nv] (a one-thread kernel of 6 us and a launch less per iteration).
 __global__ void __launch_bounds__(RB, 3) k_orth_coop(LevW lw, double* __restrict__ w,
                                                    double* __restrict__ V, long stride, int N,
                                                    const int* jd, int add, double* pa, double* pb,
                                                    unsigned* bar, int* err, double* res,
                                                    int slot_h1, int slot_h2, int slot_nrm,
-                                                   int always2) {
+                                                   int always2, ArnEnd end) {
   __shared__ double sh[(OQ + 1) * RB];
   __shared__ double h[NVMAX + 1];
   __shared__ double hu[NVMAX];
@@ -719,7 +721,10 @@ __global__ void __launch_bounds__(RB, 3) k_orth_coop(LevW lw, double* __restrict
   if (!s_re) {
     if (blockIdx.x == 0) {
       if (threadIdx.x < nv) res[slot_h2 + threadIdx.x] = 0.0;
-      if (threadIdx.x == 0) res[slot_nrm] = s_nrm;
+      if (threadIdx.x == 0) {
+        res[slot_nrm] = s_nrm;
+        if (end.c) arnoldi_end(end, hu, nullptr, s_nrm, err);
+      }
     }
     orth_final(w, V, stride, N, nv, hu, s_sc);
     return;
@@ -737,7 +742,10 @@ __global__ void __launch_bounds__(RB, 3) k_orth_coop(LevW lw, double* __restrict
   __syncthreads();
   if (blockIdx.x == 0) {
     if (threadIdx.x < nv) res[slot_h2 + threadIdx.x] = h[threadIdx.x];
-    if (threadIdx.x == 0) res[slot_nrm] = s_nrm;
+    if (threadIdx.x == 0) {
+      res[slot_nrm] = s_nrm;
+      if (end.c) arnoldi_end(end, hu, h, s_nrm, err);
+    }
   }
   orth_final(w, V, stride, N, nv, h, s_sc);
 }
@@ -884,7 +892,7 @@ LevW levw_of(const Hier& H) {
 
 int launch_cgs2_coop(const Hier& H, Reducer& R, double* w, double* V, long stride, const int* jd,
                      int add, int slot_h1, int slot_h2, int slot_nrm, cudaStream_t s,
-                     bool always2) {
+                     bool always2, const ArnEnd* arn) {
   if (R.coop_blocks <= 0) return NRD_ECUDA;
   LevW lw = levw_of(H);
   int N = H.N;
@@ -894,9 +902,10 @@ int launch_cgs2_coop(const Hier& H, Reducer& R, double* w, double* V, long strid
   int* err = R.d_err;
   double* res = R.d_res;
   int a2 = always2 ? 1 : 0;
+  ArnEnd end = arn ? *arn : ArnEnd{};
   void* args[] = {(void*)&lw, (void*)&w, (void*)&V, (void*)&stride, (void*)&N, (void*)&jd,
                   (void*)&add, (void*)&pa, (void*)&pb, (void*)&bar, (void*)&err, (void*)&res,
-                  (void*)&slot_h1, (void*)&slot_h2, (void*)&slot_nrm, (void*)&a2};
+                  (void*)&slot_h1, (void*)&slot_h2, (void*)&slot_nrm, (void*)&a2, (void*)&end};
   cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_orth_coop, dim3(R.coop_blocks),
                                               dim3(RB), args, 0, s);
   return e == cudaSuccess ? NRD_OK : NRD_ECUDA;

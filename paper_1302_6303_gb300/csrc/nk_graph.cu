@@ -35,33 +35,9 @@
 
 namespace {
 
-constexpr int kMaxTicks = 1 << 16;
 constexpr int NVMAXG = 32;
 // result slots in the reducer's device array (disjoint from solver.cu's)
 enum { G_F = 100, G_CAP = 101, G_R = 102, G_NRM = 103, G_H1 = 104, G_H2 = 140 };
-enum { NK_NAN = 1, NK_NEG = 2 };
-
-struct NkCtl {
-  double a0, dt, beta;            // read by the stencil kernels (par)
-  double fn, fn0, fold, stop, eta, tol, lam, min_lambda, gres, rn2;
-  double rtol, atol, eta_max, ew_gamma, eta0;
-  int j, total, it, krylov, flags, ticks;
-  int max_newton, max_krylov;
-  int cycles, restarts;           // executions of the cycle and restart bodies
-  int nres, nlin;                 // residual-only and linearising evaluations in the loop
-  int lin_last;                   // the last evaluation linearised (frozen J at u)
-};
-
-struct SmallG {
-  double* Hm;   // (m+1) x m, column j at Hm + (m+1) j
-  double* cs;
-  double* sn;
-  double* g;    // m+1
-  double* y;    // m
-};
-
-__device__ __forceinline__ bool tick(NkCtl* c) { return ++c->ticks < kMaxTicks; }
-
 __global__ void k_nk_params(NkCtl* c, double a0, double dt, double rtol, double atol,
                             double eta_max, double ew_gamma, double eta0, int max_newton,
                             int max_krylov, double* dbeta) {
@@ -137,37 +113,10 @@ __global__ void k_resid_g(int n, const double* F, const double* Ax, double* r) {
     r[i] = -F[i] - Ax[i];
 }
 
-// Hessenberg column j from the two CGS passes, Givens update, residual
-// estimate |g_{j+1}|; j and the iteration count advance.
-__global__ void k_arnoldi_g(NkCtl* c, SmallG S, int m, const double* res, const int* err,
-                            cudaGraphConditionalHandle hA) {
-  const int j = c->j;
-  double* col = S.Hm + (size_t)(m + 1) * j;
-  for (int i = 0; i <= j; i++) col[i] = res[G_H1 + i] + res[G_H2 + i];
-  col[j + 1] = sqrt(res[G_NRM]);
-  for (int i = 0; i < j; i++) {
-    double a = col[i], b = col[i + 1];
-    col[i] = S.cs[i] * a + S.sn[i] * b;
-    col[i + 1] = -S.sn[i] * a + S.cs[i] * b;
-  }
-  double a = col[j], b = col[j + 1];
-  double den = sqrt(a * a + b * b);
-  double cs = (den > 0.0) ? a / den : 1.0;
-  double sn = (den > 0.0) ? b / den : 0.0;
-  S.cs[j] = cs;
-  S.sn[j] = sn;
-  col[j] = den;
-  col[j + 1] = 0.0;
-  double gj = S.g[j];
-  S.g[j + 1] = -sn * gj;
-  S.g[j] = cs * gj;
-  c->gres = fabs(S.g[j + 1]);
-  c->j = j + 1;
-  c->total += 1;
-  if (!isfinite(c->gres) || *err) c->flags |= NK_NAN;
-  const bool go = tick(c) && !c->flags && c->gres > c->tol && c->j < m &&
-                  c->total < c->max_krylov;
-  cudaGraphSetConditional(hA, go ? 1u : 0u);
+// the Arnoldi step's end as a kernel of its own, where the Gram-Schmidt kernel
+// could not be launched cooperatively
+__global__ void k_arnoldi_g(ArnEnd a, const double* res, const int* err) {
+  arnoldi_end(a, res + G_H1, res + G_H2, res[G_NRM], err);
 }
 
 // Predicted convergence: a full step (lambda = 1) whose linear solve was
@@ -280,7 +229,7 @@ __global__ void k_gm_start_g(NkCtl* c, SmallG S, int m, int n, const double* __r
 __global__ void __launch_bounds__(256) k_cycle_update_g(
     NkCtl* c, SmallG S, int m, const uint8_t* __restrict__ mask, int N,
     double* __restrict__ dx, const double* __restrict__ Z, long stride,
-    const double* __restrict__ u, double* part, unsigned* counter, double* res,
+    const double* __restrict__ u, double* part, unsigned* counter, double* res, const int* err,
     cudaGraphConditionalHandle hC, cudaGraphConditionalHandle hR) {
   __shared__ double ys[NVMAXG];
   __shared__ double sh[256];
@@ -330,6 +279,7 @@ __global__ void __launch_bounds__(256) k_cycle_update_g(
       res[G_CAP] = mm;
       *counter = 0u;
       c->cycles += 1;
+      if (*err) c->flags |= NK_NAN;   // a grid barrier of the cycle gave up
       const bool conv = c->gres <= c->tol;
       const bool go = tick(c) && !conv && !c->flags && c->total < c->max_krylov;
       cudaGraphSetConditional(hC, go ? 1u : 0u);
@@ -451,14 +401,16 @@ struct Builder {
     if (r != NRD_OK) rc = r;
     jv(G->zf, c->d_w, s);
     const int* jd = &G->ctl->j;
-    if (launch_cgs2_coop(H, c->R, c->d_w, c->d_V, stride, jd, 1, G_H1, G_H2, G_NRM, s) !=
-        NRD_OK) {
+    // (the cooperative kernel ends the Arnoldi step itself)
+    const ArnEnd end = {G->ctl, small(), m, hA};
+    if (launch_cgs2_coop(H, c->R, c->d_w, c->d_V, stride, jd, 1, G_H1, G_H2, G_NRM, s, false,
+                         &end) != NRD_OK) {
       cudaGetLastError();
       launch_cgs2(H, c->R, c->d_w, c->d_V, stride, jd, 1, G_H1, G_H2, G_NRM, s);
       k_normalize_g<<<grid1(n2), 256, 0, s>>>(n2, c->d_w, c->d_V, stride, jd, 1, res() + G_NRM,
                                               1.0);
+      k_arnoldi_g<<<1, 1, 0, s>>>(end, res(), c->R.d_err);
     }
-    k_arnoldi_g<<<1, 1, 0, s>>>(G->ctl, small(), m, res(), c->R.d_err, hA);
   }
 
   // restart from the true residual (body of the IF node)
@@ -516,7 +468,7 @@ struct Builder {
     // last cycle's stands), the cycle-end test
     k_cycle_update_g<<<c->R.nblk, 256, 0, s>>>(G->ctl, small(), c->kry_m, c->H.d_mask, c->H.N,
                                                c->d_dx, c->d_Z, n2, G->uw, c->R.d_part,
-                                               c->R.d_count, res(), hC, hR);
+                                               c->R.d_count, res(), c->R.d_err, hC, hR);
   }
 
   // the Newton loop body

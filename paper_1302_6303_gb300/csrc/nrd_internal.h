@@ -83,7 +83,6 @@ struct Hier {
   int* d_rf_off = nullptr;                // nrf+1, entries per cell
   int* d_rf_face = nullptr;               // entries: face 0..5 of the coarse cell
   int4* d_rf_g = nullptr;                 // entries: ghost slots of the 4 fine fluxes
-  int* d_rf_level = nullptr;              // nrf: level of the coarse cell
   int rf_lstart[NRD_MAX_LEVELS + 1] = {}; // first entry of each level (cells ascend by level)
   // transposed ghost stencils (adjoint): cell -> (ghost, weight), and the
   // sibling / coarse-fine ghosts that take their z from a cell
@@ -243,10 +242,12 @@ void launch_cgs2(const Hier& H, Reducer& R, double* w, const double* V, long str
 // reduction in the common case, two otherwise; norms by the Pythagorean
 // identity), writing V[nv] = w' / |w'|.  For vectors that vanish on covered
 // cells.  always2: the second pass every time (CGS2).
+// end: the kernel also ends the Arnoldi step of the Newton graph (arnoldi_end).
 // Returns NRD_ECUDA if a cooperative launch is not possible.
+struct ArnEnd;
 int launch_cgs2_coop(const Hier& H, Reducer& R, double* w, double* V, long stride, const int* jd,
                      int add, int slot_h1, int slot_h2, int slot_nrm, cudaStream_t s,
-                     bool always2 = false);
+                     bool always2 = false, const ArnEnd* end = nullptr);
 
 // Preconditioner (k_pc.cu)
 struct PcState;
@@ -400,6 +401,76 @@ int ctx_linearise(nrd_ctx* c, const double* u, const double* b, double a0, doubl
                   cudaStream_t s, const double* par = nullptr, bool with_dz = false);
 
 #ifdef __CUDACC__
+// ---- control block of the Newton graph (nk_graph.cu); the end of an Arnoldi
+// step is shared with the cooperative Gram-Schmidt kernel (k_blas.cu)
+constexpr int kMaxTicks = 1 << 16;
+enum { NK_NAN = 1, NK_NEG = 2 };
+
+struct NkCtl {
+  double a0, dt, beta;            // read by the stencil kernels (par)
+  double fn, fn0, fold, stop, eta, tol, lam, min_lambda, gres, rn2;
+  double rtol, atol, eta_max, ew_gamma, eta0;
+  int j, total, it, krylov, flags, ticks;
+  int max_newton, max_krylov;
+  int cycles, restarts;           // executions of the cycle and restart bodies
+  int nres, nlin;                 // residual-only and linearising evaluations in the loop
+  int lin_last;                   // the last evaluation linearised (frozen J at u)
+};
+
+struct SmallG {
+  double* Hm;   // (m+1) x m, column j at Hm + (m+1) j
+  double* cs;
+  double* sn;
+  double* g;    // m+1
+  double* y;    // m
+};
+
+__device__ __forceinline__ bool tick(NkCtl* c) { return ++c->ticks < kMaxTicks; }
+
+// what the end of an Arnoldi step updates
+struct ArnEnd {
+  NkCtl* c;
+  SmallG S;
+  int m;
+  cudaGraphConditionalHandle hA;
+};
+
+// Hessenberg column j from the two Gram-Schmidt passes (h1, h2) and the squared
+// norm, Givens update, residual estimate |g_{j+1}|; j and the iteration count
+// advance.  One thread.
+__device__ __forceinline__ void arnoldi_end(const ArnEnd& a, const double* h1, const double* h2,
+                                            double nrm, const int* err) {
+  NkCtl* c = a.c;
+  const SmallG& S = a.S;
+  const int m = a.m, j = c->j;
+  double* col = S.Hm + (size_t)(m + 1) * j;
+  for (int i = 0; i <= j; i++) col[i] = h1[i] + (h2 ? h2[i] : 0.0);
+  col[j + 1] = sqrt(nrm);
+  for (int i = 0; i < j; i++) {
+    double x = col[i], y = col[i + 1];
+    col[i] = S.cs[i] * x + S.sn[i] * y;
+    col[i + 1] = -S.sn[i] * x + S.cs[i] * y;
+  }
+  double x = col[j], y = col[j + 1];
+  double den = sqrt(x * x + y * y);
+  double cs = (den > 0.0) ? x / den : 1.0;
+  double sn = (den > 0.0) ? y / den : 0.0;
+  S.cs[j] = cs;
+  S.sn[j] = sn;
+  col[j] = den;
+  col[j + 1] = 0.0;
+  double gj = S.g[j];
+  S.g[j + 1] = -sn * gj;
+  S.g[j] = cs * gj;
+  c->gres = fabs(S.g[j + 1]);
+  c->j = j + 1;
+  c->total += 1;
+  if (!isfinite(c->gres) || *err) c->flags |= NK_NAN;
+  const bool go = tick(c) && !c->flags && c->gres > c->tol && c->j < m &&
+                  c->total < c->max_krylov;
+  cudaGraphSetConditional(a.hA, go ? 1u : 0u);
+}
+
 // Candidate test of the positivity cap (Sec. 4.1 remark: lambda =
 // min(1, 0.9 min over x_i < 0 of u_i / (-x_i))): true when x < 0 (not -0, not
 // NaN) and u / (-x) may be below 2, read from the exponent fields with integer
