@@ -326,7 +326,9 @@ int nrd_tag(nrd_ctx* ctx, const double* u, double thr_c, double thr_g, double th
  *   last), boxes_out[6*max_boxes] inclusive lo/hi per box in layout order
  *   (level 0 is the base box), *total_out the total box count (also set when
  *   it exceeds max_boxes, which returns NRD_EINVAL, as does a level whose
- *   index space has 2^31 cells or more).  Synchronises. */
+ *   index space has 2^31 cells or more).  The fields of a level (about 14 bytes
+ *   per cell of its index space) are formed in device memory, on the host when
+ *   that is not to be had.  Synchronises. */
 int nrd_regrid_boxes(nrd_ctx* ctx, const uint8_t* tags, int tag_bits, int buffer,
                      double efficiency, int min_side, int max_side, int max_levels,
                      int max_boxes, int* nlevels_out, int* nboxes_out, int* boxes_out,
@@ -342,12 +344,12 @@ int nrd_regrid_boxes(nrd_ctx* ctx, const uint8_t* tags, int tag_bits, int buffer
  * leaf sums of V u are conserved and no value leaves the range of the old
  * neighbours (E, T stay positive).
  *   u_src: device, nvec x 2*ncells(src) doubles;  u_dst: device,
- *   nvec x 2*ncells(dst) doubles (every cell written).  Allocates and frees
- *   one device buffer: a copy of u_src, 4 bytes per new cell (the old cell it
- *   copies, or -1) and 44 bytes per reconstructed cell (the source list is
- *   built on host threads).  Synchronises.
+ *   nvec x 2*ncells(dst) doubles (every cell written).  Where the old
+ * hierarchy has finer levels, ctx_src holds a device buffer for it: a copy of
+ * u_src and 4 bytes per cell of the level below the finest (kept up to 256 MB,
+ * else freed before the call returns).  Synchronises.
  * Errors: NRD_ESTATE (a context without hierarchy), NRD_EINVAL (different
- * base grids, null pointers, nvec < 1, a new cell in no old cell),
+ * base grids, null pointers, nvec < 1),
  * NRD_ENOMEM, NRD_ECUDA; the message is stored in ctx_dst. */
 int nrd_transfer(nrd_ctx* ctx_src, nrd_ctx* ctx_dst, const double* u_src, double* u_dst,
                  int nvec, cudaStream_t stream);

@@ -86,7 +86,9 @@ void set_model(nrd_ctx* c) {
 void free_fields(nrd_ctx* c) {
   auto F = [](void* p) { if (p) cudaFree(p); };
   F(c->d_z); F(c->d_gz); F(c->d_gu); F(c->d_gv); F(c->d_cf); F(c->d_tmp); F(c->jac.jc); F(c->d_pef);
-  F(c->d_gam); F(c->d_z3);
+  F(c->d_gam); F(c->d_z3); F(c->d_xfer);
+  c->d_xfer = nullptr;
+  c->xfer_bytes = 0;
   c->jac = Jac();
   c->d_z3 = nullptr;
   c->d_z = nullptr; c->d_gz = nullptr; c->d_gu = nullptr; c->d_gv = nullptr; c->d_cf = nullptr;

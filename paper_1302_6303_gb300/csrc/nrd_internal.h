@@ -331,6 +331,8 @@ struct nrd_ctx {
   double* d_gv = nullptr;      // 2G: ghosts of a direction
   double* d_cf = nullptr;      // 2G: fine-side coarse-fine fluxes
   double* d_tmp = nullptr;     // 2N scratch
+  void* d_xfer = nullptr;      // scratch of nrd_regrid_boxes and nrd_transfer (regrid.cu)
+  size_t xfer_bytes = 0;
   Jac jac;                     // frozen Jacobian (one allocation, at jac.jc)
   double* d_pef = nullptr;     // [2][3N+G] face fluxes of the split linearisation
   double* d_gam = nullptr;     // [3][G] adjoint ghost scratch

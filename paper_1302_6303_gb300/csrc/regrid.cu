@@ -24,9 +24,13 @@
 // Accepted boxes, refined by 2, are the boxes of level l+1, in the order the
 // recursion accepts them (lower part first).
 //
+// The tagged and nestable fields of a level and their summed-area tables are
+// formed on the device (scatter, box filters, scans); the recursion reads the
+// tables on the host, 8 entries per count.
+//
 // nrd_transfer: conservative limited-linear transfer of state vectors from an
-// old to a new hierarchy (device gather; the per-cell source list is built on
-// host threads).  The
+// old to a new hierarchy, one device kernel that looks every new cell's source
+// up in the old hierarchy's maps.  The
 // old vectors are first made composite (covered cells := mean of their
 // children).  A new cell that exists on the same level of the old hierarchy
 // copies it; any other new cell evaluates, at its centre, the limited linear
@@ -42,7 +46,6 @@
 #include <cstdint>
 #include <cstring>
 #include <string>
-#include <thread>
 #include <vector>
 
 #include "nrd_internal.h"
@@ -101,14 +104,18 @@ void box_filter(std::vector<uint8_t>& v, const int n[3], int d, int r, bool take
 }
 
 // Counts over boxes in O(1): a summed-area table of a dense 0/1 field,
-// S(i, j, k) = number of set cells in [0, i) x [0, j) x [0, k).
+// S(i, j, k) = number of set cells in [0, i) x [0, j) x [0, k); without a table
+// every cell is set.
 struct BoxSum {
   int n[3];
-  std::vector<int> S;
-  BoxSum(const std::vector<uint8_t>& v, const int nn[3]) {
+  const int* S;
+  BoxSum(const int* table, const int nn[3]) : S(table) {
     for (int d = 0; d < 3; d++) n[d] = nn[d];
+  }
+  // the table of a host field
+  static std::vector<int> table(const std::vector<uint8_t>& v, const int n[3]) {
     const long sx = n[0] + 1, sxy = sx * (n[1] + 1);
-    S.assign(sxy * (n[2] + 1), 0);
+    std::vector<int> S(sxy * (n[2] + 1), 0);
     for (int k = 0; k < n[2]; k++)
       for (int j = 0; j < n[1]; j++) {
         const uint8_t* row = &v[(long)n[0] * (j + (long)n[1] * k)];
@@ -122,8 +129,10 @@ struct BoxSum {
           o[i + 1] = line + dn[i + 1] + bk[i + 1] - db[i + 1];
         }
       }
+    return S;
   }
   long count(const int lo[3], const int hi[3]) const {
+    if (!S) return (long)(hi[0] - lo[0] + 1) * (hi[1] - lo[1] + 1) * (hi[2] - lo[2] + 1);
     const long sx = n[0] + 1, sxy = sx * (n[1] + 1);
     auto at = [&](int i, int j, int k) { return (long)S[k * sxy + j * sx + i]; };
     const int a0 = lo[0], a1 = lo[1], a2 = lo[2], b0 = hi[0] + 1, b1 = hi[1] + 1, b2 = hi[2] + 1;
@@ -245,46 +254,277 @@ struct Clusterer {
   }
 };
 
-// A new cell that is not a copy of an old cell on its own level: the old
-// coarse cell src, its six neighbours on that level (-1: none; x-, x+, y-,
-// ...) and the new cell centre relative to src's, (x - x_c) / h_c per axis
-// (a multiple of 1/2^(l - lc + 1), exact in float).
-struct ReconDesc {
-  int cell;         // the new cell
-  int src;
-  int nb[6];
-  float off[3];
+// ---- device side of the clustering: dense fields of one level
+struct Dims {
+  int n0, n1, n2;
+  __device__ long at(int i, int j, int k) const { return i + (long)n0 * (j + (long)n1 * k); }
 };
 
+// raw[q] := tag of the level-lc cell holding q, for every level-lc cell of the
+// current hierarchy; called from the coarsest level to min(l, finest), so that
+// the finest cell's tag stays.  Grid (patches, blocks per patch).
+__global__ void k_rg_scatter(const PatchDev* __restrict__ patches, const uint8_t* __restrict__ tags,
+                             int bits, int shift, Dims D, uint8_t* __restrict__ raw) {
+  const PatchDev P = patches[blockIdx.x];
+  const int nc = P.n[0] * P.n[1] * P.n[2], r = 1 << shift;
+  for (int c = blockIdx.y * blockDim.x + threadIdx.x; c < nc; c += gridDim.y * blockDim.x) {
+    const int q = c / P.n[0], i = P.lo[0] + c - q * P.n[0];
+    const int k = q / P.n[1], j = P.lo[1] + q - k * P.n[1], kk = P.lo[2] + k;
+    const uint8_t t = (tags[P.off + c] & bits) ? 1 : 0;
+    for (int z = 0; z < r; z++)
+      for (int y = 0; y < r; y++)
+        for (int x = 0; x < r; x++) raw[D.at(i * r + x, j * r + y, kk * r + z)] = t;
+  }
+}
+
+// in[q] := 1 on the boxes of the new level.  Grid (boxes, blocks per box).
+__global__ void k_rg_boxes(const int* __restrict__ boxes, Dims D, uint8_t* __restrict__ in) {
+  const int* b = boxes + 6 * blockIdx.x;
+  const int s0 = b[3] - b[0] + 1, s1 = b[4] - b[1] + 1, nc = s0 * s1 * (b[5] - b[2] + 1);
+  for (int c = blockIdx.y * blockDim.x + threadIdx.x; c < nc; c += gridDim.y * blockDim.x) {
+    const int q = c / s0, k = q / s1;
+    in[D.at(b[0] + c - q * s0, b[1] + q - k * s1, b[2] + k)] = 1;
+  }
+}
+
+// one axis of the box filters: hit := OR of raw within r cells (of cells that
+// are in the level, where in is given), ok := AND of in within 1 cell, both
+// inside the domain.  first: the x axis, where raw counts on the level only.
+__global__ void k_rg_filter(Dims D, int axis, int r, bool first, const uint8_t* __restrict__ raw,
+                            const uint8_t* __restrict__ in0, const uint8_t* __restrict__ in,
+                            uint8_t* __restrict__ hit, uint8_t* __restrict__ ok) {
+  const long nn = (long)D.n0 * D.n1 * D.n2;
+  const long st = axis == 0 ? 1 : (axis == 1 ? (long)D.n0 : (long)D.n0 * D.n1);
+  const int m = axis == 0 ? D.n0 : (axis == 1 ? D.n1 : D.n2);
+  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < nn;
+       q += (long)gridDim.x * blockDim.x) {
+    const int x = (int)((q / st) % m);
+    uint8_t h = 0;
+    for (int d = -min(r, x); d <= min(r, m - 1 - x); d++) {
+      const uint8_t v = raw[q + d * st];
+      h |= (first && in0) ? (v & in0[q + d * st]) : v;
+    }
+    hit[q] = h;
+    if (in) {
+      uint8_t o = in[q];
+      if (x > 0) o &= in[q - st];
+      if (x < m - 1) o &= in[q + st];
+      ok[q] = o;
+    }
+  }
+}
+
+// Summed-area tables of the tagged field (tag on nestable cells) and, where
+// there is one, the nestable field (blockIdx.y = 1): first the rows (one warp
+// each, a scan per 32 cells), then running sums along y and z.  S: tables of
+// (n0 + 1)(n1 + 1)(n2 + 1) entries, one after the other, zeroed.
+__global__ void k_rg_rows(Dims D, const uint8_t* __restrict__ hit, const uint8_t* __restrict__ ok,
+                          int* __restrict__ S) {
+  const long sx = D.n0 + 1, sxy = sx * (D.n1 + 1), tab = sxy * (D.n2 + 1);
+  const int f = blockIdx.y, lane = threadIdx.x & 31;
+  const long rows = (long)D.n1 * D.n2;
+  for (long w = (blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5; w < rows;
+       w += ((long)gridDim.x * blockDim.x) >> 5) {
+    const int j = (int)(w % D.n1), k = (int)(w / D.n1);
+    int* o = S + f * tab + (k + 1) * sxy + (j + 1) * sx + 1;
+    int base = 0;
+    for (int i0 = 0; i0 < D.n0; i0 += 32) {
+      const int i = i0 + lane;
+      int v = 0;
+      if (i < D.n0) {
+        const long q = D.at(i, j, k);
+        const uint8_t a = ok ? ok[q] : 1;
+        v = f ? a : (a & hit[q]);
+      }
+      for (int s = 1; s < 32; s <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, s);
+        if (lane >= s) v += u;
+      }
+      if (i < D.n0) o[i] = base + v;
+      base += __shfl_sync(0xffffffffu, v, 31);
+    }
+  }
+}
+// axis 1: along y for every (i, k); axis 2: along z for every (i, j)
+__global__ void k_rg_sums(Dims D, int axis, int* __restrict__ S) {
+  const long sx = D.n0 + 1, sxy = sx * (D.n1 + 1), tab = sxy * (D.n2 + 1);
+  const int other = axis == 1 ? D.n2 : D.n1, m = axis == 1 ? D.n1 : D.n2;
+  const long so = axis == 1 ? sxy : sx, st = axis == 1 ? sx : sxy;
+  const long lines = (long)D.n0 * other;
+  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < lines;
+       t += (long)gridDim.x * blockDim.x) {
+    int* p = S + blockIdx.y * tab + (t % D.n0) + 1 + (t / D.n0 + 1) * so + st;
+    int acc = 0;
+#pragma unroll 8
+    for (int x = 0; x < m; x++, p += st) {
+      acc += *p;
+      *p = acc;
+    }
+  }
+}
+
+int rg_blocks(long n) { return (int)std::max(1L, std::min(152L * 8, (n + 255) / 256)); }
+
+// Device scratch of a context for the two calls here, both of which synchronise
+// before they return: kept up to kKeep bytes (an allocation and its release
+// cost more than the kernels of a 64^3 level: 170 of 400 us), else given back by
+// xfer_done.  null when the allocation fails.
+constexpr size_t kKeep = 256u << 20;
+void* xfer_reserve(nrd_ctx* c, size_t bytes) {
+  if (bytes > c->xfer_bytes) {
+    if (c->d_xfer) cudaFree(c->d_xfer);
+    c->d_xfer = nullptr;
+    c->xfer_bytes = 0;
+    if (cudaMalloc(&c->d_xfer, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      c->d_xfer = nullptr;
+      return nullptr;
+    }
+    c->xfer_bytes = bytes;
+  }
+  return c->d_xfer;
+}
+void xfer_done(nrd_ctx* c) {
+  if (c->xfer_bytes <= kKeep) return;
+  cudaFree(c->d_xfer);
+  c->d_xfer = nullptr;
+  c->xfer_bytes = 0;
+}
+
+// the device fields and tables of one level
+struct RgDevice {
+  nrd_ctx* c;
+  ~RgDevice() { xfer_done(c); }
+  // tables of the tagged cells and (unless the level covers the domain) of the
+  // nestable cells, on the host; false when the device had no memory for it
+  bool tables(const Hier& H, const uint8_t* tags, int bits, int buffer, int l, const int n[3],
+              const std::vector<IBox>& boxes, std::vector<int>& S, cudaError_t& e) {
+    const long nn = (long)n[0] * n[1] * n[2];
+    const long tab = (long)(n[0] + 1) * (n[1] + 1) * (n[2] + 1);
+    const bool full = l == 0;                      // one box: the whole domain
+    const int nt = full ? 1 : 2;
+    const size_t pad = (nn + 255) / 256 * 256;
+    const size_t bytes = 6 * pad + nt * tab * sizeof(int) + 6 * boxes.size() * sizeof(int);
+    uint8_t* buf = (uint8_t*)xfer_reserve(c, bytes);
+    if (!buf) return false;
+    uint8_t *raw = buf, *in = raw + pad, *h1 = in + pad, *o1 = h1 + pad, *h2 = o1 + pad,
+            *o2 = h2 + pad;
+    int* dS = (int*)(buf + 6 * pad);
+    int* dB = dS + nt * tab;
+    const Dims D{n[0], n[1], n[2]};
+    for (int lc = 0; lc <= std::min(l, H.L - 1); lc++) {
+      const LevelInfo& Lv = H.lev[lc];
+      const int per = (int)std::max(1L, std::min(152L * 8L / Lv.np + 1, (Lv.ncell / Lv.np + 255L) / 256));
+      k_rg_scatter<<<dim3(Lv.np, per), 256>>>(H.d_patches + Lv.p0, tags, bits, l - lc, D, raw);
+    }
+    if (!full) {
+      std::vector<int> hb;
+      for (const IBox& b : boxes) {
+        hb.insert(hb.end(), b.lo, b.lo + 3);
+        hb.insert(hb.end(), b.hi, b.hi + 3);
+      }
+      cudaMemcpy(dB, hb.data(), hb.size() * sizeof(int), cudaMemcpyHostToDevice);
+      cudaMemsetAsync(in, 0, nn);
+      k_rg_boxes<<<dim3((unsigned)boxes.size(), 8), 256>>>(dB, D, in);
+    }
+    cudaMemsetAsync(dS, 0, nt * tab * sizeof(int));
+    const int g = rg_blocks(nn);
+    const uint8_t* i0 = full ? nullptr : in;
+    k_rg_filter<<<g, 256>>>(D, 0, buffer, true, raw, i0, i0, h1, o1);
+    k_rg_filter<<<g, 256>>>(D, 1, buffer, false, h1, nullptr, full ? nullptr : o1, h2, o2);
+    k_rg_filter<<<g, 256>>>(D, 2, buffer, false, h2, nullptr, full ? nullptr : o2, h1, o1);
+    k_rg_rows<<<dim3(rg_blocks((long)n[1] * n[2] * 32), nt), 256>>>(D, h1, full ? nullptr : o1, dS);
+    k_rg_sums<<<dim3(rg_blocks((long)n[0] * n[2]), nt), 256>>>(D, 1, dS);
+    k_rg_sums<<<dim3(rg_blocks((long)n[0] * n[1]), nt), 256>>>(D, 2, dS);
+    S.resize(nt * tab);
+    e = cudaMemcpy(S.data(), dS, nt * tab * sizeof(int), cudaMemcpyDeviceToHost);
+    return true;
+  }
+};
+
+// ---- transfer
 __device__ __forceinline__ double minmod(double a, double b) {
   if (a * b <= 0.0) return 0.0;
   return (fabs(a) < fabs(b)) ? a : b;
 }
 
-// Threads [0, N): new cells with code >= 0 copy old cell code for every
-// field.  Threads [N, N + nrec): the reconstruction entries.
-__global__ void k_transfer(const int* __restrict__ code, const ReconDesc* __restrict__ rec,
-                           int N, int nrec, int Nold, int nvec, const double* __restrict__ uo,
-                           double* __restrict__ un) {
-  const long total = (long)N + nrec;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
-       t += (long)gridDim.x * blockDim.x) {
-    if (t < N) {
-      const int src = code[t];
-      if (src < 0) continue;
-      for (int f = 0; f < 2 * nvec; f++) un[(long)f * N + t] = uo[(long)f * Nold + src];
+// The old hierarchy's cell look-up: dense maps up to the level below the
+// finest; a finest cell is the child of a covered cell there (slot: index of
+// a level L - 2 cell in the covered list, or -1).  One level: the box itself.
+struct OldCells {
+  int L;
+  int n[NRD_MAX_LEVELS][3];
+  const int* lmap[NRD_MAX_LEVELS];
+  const int4* cov;
+  const int* slot;
+  int off;                       // first cell of level L - 2
+  __device__ int find(int l, int x, int y, int z) const {
+    if (l >= L || x < 0 || y < 0 || z < 0 || x >= n[l][0] || y >= n[l][1] || z >= n[l][2])
+      return -1;
+    if (l == 0 && L == 1) return x + n[0][0] * (y + n[0][1] * z);
+    if (l < L - 1) return lmap[l][x + (long)n[l][0] * (y + (long)n[l][1] * z)];
+    const int p = lmap[l - 1][(x >> 1) + (long)n[l - 1][0] * ((y >> 1) + (long)n[l - 1][1] * (z >> 1))];
+    if (p < 0) return -1;
+    const int e = slot[p - off];
+    if (e < 0) return -1;
+    const int4 c = cov[e];
+    return c.y + (x & 1) + (y & 1) * c.z + (z & 1) * c.w;
+  }
+};
+
+__global__ void k_cov_slots(const int4* __restrict__ cov, int n, int off, int* __restrict__ slot) {
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x)
+    slot[cov[q].x - off] = q;
+}
+
+// One new cell per thread over the new hierarchy's tiles: a cell that exists on
+// its level of the old hierarchy is copied, any other takes the limited linear
+// reconstruction of the finest old cell holding it.
+__global__ void k_transfer(const TileDev* __restrict__ tiles, const PatchDev* __restrict__ patches,
+                           int tx, int ty, OldCells O, int N, int Nold, int nvec,
+                           const double* __restrict__ uo, double* __restrict__ un) {
+  const TileDev tile = tiles[blockIdx.x];
+  const PatchDev P = patches[tile.patch];
+  const int ex = min(tx, P.n[0] - tile.i0), ey = min(ty, P.n[1] - tile.j0);
+  const int nc = ex * ey * (tile.k1 - tile.k0), l = P.level;
+  for (int t = threadIdx.x; t < nc; t += blockDim.x) {
+    const int r0 = t / ex, i = tile.i0 + t - r0 * ex;
+    const int rk = r0 / ey, j = tile.j0 + r0 - rk * ey, k = tile.k0 + rk;
+    const int c = P.off + i + P.n[0] * (j + P.n[1] * k);
+    const int q[3] = {P.lo[0] + i, P.lo[1] + j, P.lo[2] + k};
+    int lc = min(l, O.L - 1), src = -1, cq[3] = {0, 0, 0};
+    for (; lc >= 0; lc--) {
+      for (int d = 0; d < 3; d++) cq[d] = q[d] >> (l - lc);
+      src = O.find(lc, cq[0], cq[1], cq[2]);
+      if (src >= 0) break;
+    }
+    if (lc == l) {
+      for (int f = 0; f < 2 * nvec; f++) un[(long)f * N + c] = uo[(long)f * Nold + src];
       continue;
     }
-    const ReconDesc r = rec[t - N];
+    // (the base level covers the domain, so src >= 0)
+    const int r = 1 << (l - lc);
+    int nb[6];
+    double off[3];
+    for (int d = 0; d < 3; d++) {
+      // centre of the new cell relative to the old one, in old cells (a
+      // multiple of 1/2^(l - lc + 1), exact)
+      off[d] = (2.0 * (q[d] - cq[d] * r) + 1.0 - r) / (2.0 * r);
+      for (int sd = 0; sd < 2; sd++) {
+        int nq[3] = {cq[0], cq[1], cq[2]};
+        nq[d] += sd ? 1 : -1;
+        nb[2 * d + sd] = O.find(lc, nq[0], nq[1], nq[2]);
+      }
+    }
     for (int f = 0; f < 2 * nvec; f++) {
       const double* u = uo + (long)f * Nold;
-      const double uc = u[r.src];
+      const double uc = u[src];
       double v = uc;
       for (int a = 0; a < 3; a++) {
-        const int im = r.nb[2 * a], ip = r.nb[2 * a + 1];
-        if (im >= 0 && ip >= 0) v += minmod(uc - u[im], u[ip] - uc) * (double)r.off[a];
+        const int im = nb[2 * a], ip = nb[2 * a + 1];
+        if (im >= 0 && ip >= 0) v += minmod(uc - u[im], u[ip] - uc) * off[a];
       }
-      un[(long)f * N + r.cell] = v;
+      un[(long)f * N + c] = v;
     }
   }
 }
@@ -311,11 +551,7 @@ int nrd_regrid_boxes(nrd_ctx* c, const uint8_t* tags, int tag_bits, int buffer,
     return NRD_EINVAL;
   }
   const Hier& H = c->H;
-  std::vector<uint8_t> htags(H.N);
-  if (cudaMemcpy(htags.data(), tags, H.N, cudaMemcpyDeviceToHost) != cudaSuccess) {
-    c->err = "copy of the tags failed";
-    return NRD_ECUDA;
-  }
+  std::vector<uint8_t> htags;   // filled when a level is done on the host
   const int n0[3] = {H.lev[0].n[0], H.lev[0].n[1], H.lev[0].n[2]};
   // tag of the current cell (l, q), or -1 if the current hierarchy has none
   auto cur_tag = [&](int l, const int q[3]) -> int {
@@ -333,33 +569,58 @@ int nrd_regrid_boxes(nrd_ctx* c, const uint8_t* tags, int tag_bits, int buffer,
       c->err = "nrd_regrid_boxes: a level is too large for int32 box counts";
       return NRD_EINVAL;
     }
-    auto li = [&](int i, int j, int k) { return i + (long)n[0] * (j + (long)n[1] * k); };
-    std::vector<uint8_t> in(lsize, 0), raw(lsize, 0), tg(lsize, 0), ok(lsize, 0);
-    for (const IBox& b : levels[l])
-      for (int k = b.lo[2]; k <= b.hi[2]; k++)
-        for (int j = b.lo[1]; j <= b.hi[1]; j++)
-          for (int i = b.lo[0]; i <= b.hi[0]; i++) {
-            in[li(i, j, k)] = 1;
-            int t = -1;
-            for (int lc = std::min(l, H.L - 1); lc >= 0 && t < 0; lc--) {
-              const int q[3] = {i >> (l - lc), j >> (l - lc), k >> (l - lc)};
-              t = cur_tag(lc, q);
+    // on the device; on the host where its memory does not allow the fields
+    std::vector<int> tables, osum_h;
+    RgDevice dev{c};
+    cudaError_t e = cudaSuccess;
+    const bool on_device = dev.tables(H, tags, tag_bits, buffer, l, n, levels[l], tables, e);
+    if (on_device && (e != cudaSuccess || cudaGetLastError() != cudaSuccess)) {
+      c->err = "clustering kernels failed";
+      return NRD_ECUDA;
+    }
+    const int* ttab = tables.data();
+    const int* otab = nullptr;   // null: every cell is nestable
+    if (on_device && l > 0) otab = tables.data() + (long)(n[0] + 1) * (n[1] + 1) * (n[2] + 1);
+    if (!on_device) {
+      if (htags.empty()) {
+        htags.resize(H.N);
+        if (cudaMemcpy(htags.data(), tags, H.N, cudaMemcpyDeviceToHost) != cudaSuccess) {
+          c->err = "copy of the tags failed";
+          return NRD_ECUDA;
+        }
+      }
+      auto li = [&](int i, int j, int k) { return i + (long)n[0] * (j + (long)n[1] * k); };
+      std::vector<uint8_t> in(lsize, 0), raw(lsize, 0), tg(lsize, 0), ok(lsize, 0);
+      for (const IBox& b : levels[l])
+        for (int k = b.lo[2]; k <= b.hi[2]; k++)
+          for (int j = b.lo[1]; j <= b.hi[1]; j++)
+            for (int i = b.lo[0]; i <= b.hi[0]; i++) {
+              in[li(i, j, k)] = 1;
+              int t = -1;
+              for (int lc = std::min(l, H.L - 1); lc >= 0 && t < 0; lc--) {
+                const int q[3] = {i >> (l - lc), j >> (l - lc), k >> (l - lc)};
+                t = cur_tag(lc, q);
+              }
+              raw[li(i, j, k)] = t > 0 ? 1 : 0;
             }
-            raw[li(i, j, k)] = t > 0 ? 1 : 0;
-          }
-    // ok: every neighbour of the 3x3x3 block inside the domain is in the new
-    // level (proper nesting); tg: a raw tag within `buffer` cells (inside the
-    // domain), on ok cells.  Both are box filters, done one axis at a time:
-    // the minimum of `in` over windows of 3 (outside the domain counts as
-    // in), the maximum of `raw` over windows of 2 buffer + 1 (outside counts
-    // as untagged).
-    ok = in;
-    for (int d = 0; d < 3; d++) box_filter(ok, n, d, 1, true);
-    std::vector<uint8_t> hit = raw;
-    for (int d = 0; d < 3; d++) box_filter(hit, n, d, buffer, false);
-    for (long q = 0; q < lsize; q++) tg[q] = (ok[q] && hit[q]) ? 1 : 0;
+      // ok: every neighbour of the 3x3x3 block inside the domain is in the new
+      // level (proper nesting); tg: a raw tag within `buffer` cells (inside the
+      // domain), on ok cells.  Both are box filters, done one axis at a time:
+      // the minimum of `in` over windows of 3 (outside the domain counts as
+      // in), the maximum of `raw` over windows of 2 buffer + 1 (outside counts
+      // as untagged).
+      ok = in;
+      for (int d = 0; d < 3; d++) box_filter(ok, n, d, 1, true);
+      std::vector<uint8_t> hit = raw;
+      for (int d = 0; d < 3; d++) box_filter(hit, n, d, buffer, false);
+      for (long q = 0; q < lsize; q++) tg[q] = (ok[q] && hit[q]) ? 1 : 0;
+      tables = BoxSum::table(tg, n);
+      osum_h = BoxSum::table(ok, n);
+      ttab = tables.data();
+      otab = osum_h.data();
+    }
     std::vector<IBox> coarse;
-    const BoxSum tsum(tg, n), osum(ok, n);
+    const BoxSum tsum(ttab, n), osum(otab, n);
     Clusterer C{tsum, osum, {n[0], n[1], n[2]}, efficiency, max_side / 2, min_side / 2, coarse};
     C.run(IBox{{0, 0, 0}, {n[0] - 1, n[1] - 1, n[2] - 1}});
     if (coarse.empty()) break;
@@ -414,110 +675,44 @@ int nrd_transfer(nrd_ctx* src, nrd_ctx* dst, const double* u_src, double* u_dst,
       dst->err = "the hierarchies have different base grids";
       return NRD_EINVAL;
     }
-  auto old_cell = [&](int l, const int q[3]) -> int {
-    if (l < 0 || l >= A.L) return -1;
-    for (int d = 0; d < 3; d++)
-      if (q[d] < 0 || q[d] >= A.lev[l].n[d]) return -1;
-    return A.lmap[l][q[0] + (long)A.lev[l].n[0] * (q[1] + (long)A.lev[l].n[1] * q[2])];
-  };
-  // Per new cell: the old cell on the same level (a copy), else -1 and a
-  // reconstruction entry.  Patches are split over host threads; each thread
-  // keeps its own entries, concatenated afterwards.
-  std::vector<int> code(B.N);
-  const int np = (int)B.patches.size();
-  int nth = (int)std::min<long>(16, std::max<long>(1, (long)B.N / 65536));
-  nth = std::max(1, std::min(nth, (int)std::thread::hardware_concurrency()));
-  std::vector<std::vector<ReconDesc>> recs(nth);
-  std::vector<int> fail(nth, 0);
-  auto work = [&](int th) {
-    // patches of thread th: a contiguous range holding about 1/nth of the cells
-    const long lo_cell = (long)B.N * th / nth, hi_cell = (long)B.N * (th + 1) / nth;
-    for (int p = 0; p < np; p++) {
-      const PatchDev& P = B.patches[p];
-      if (P.off < lo_cell || P.off >= hi_cell) continue;
-      const int l = P.level;
-      for (int k = 0; k < P.n[2]; k++)
-        for (int j = 0; j < P.n[1]; j++)
-          for (int i = 0; i < P.n[0]; i++) {
-            const int q[3] = {P.lo[0] + i, P.lo[1] + j, P.lo[2] + k};
-            const int c = P.off + i + P.n[0] * (j + P.n[1] * k);
-            code[c] = old_cell(l, q);
-            if (code[c] >= 0) continue;
-            int lc = std::min(l, A.L) - 1, cq[3] = {0, 0, 0};
-            for (; lc >= 0; lc--) {
-              for (int d = 0; d < 3; d++) cq[d] = q[d] >> (l - lc);
-              if (old_cell(lc, cq) >= 0) break;
-            }
-            if (lc < 0) {
-              fail[th] = 1;
-              return;
-            }
-            ReconDesc t;
-            t.cell = c;
-            t.src = old_cell(lc, cq);
-            const int r = 1 << (l - lc);
-            for (int d = 0; d < 3; d++) {
-              // centre of the new cell relative to the old one, in old cells
-              t.off[d] = (float)((2.0 * (q[d] - cq[d] * r) + 1.0 - r) / (2.0 * r));
-              for (int sd = 0; sd < 2; sd++) {
-                int nq[3] = {cq[0], cq[1], cq[2]};
-                nq[d] += sd ? 1 : -1;
-                t.nb[2 * d + sd] = old_cell(lc, nq);
-              }
-            }
-            recs[th].push_back(t);
-          }
-    }
-  };
-  if (nth == 1) {
-    work(0);
-  } else {
-    // a part whose thread cannot be started (the system refuses it) runs here
-    std::vector<std::thread> pool;
-    int started = 0;
-    try {
-      for (; started < nth; started++) pool.emplace_back(work, started);
-    } catch (...) {
-    }
-    for (int th = started; th < nth; th++) work(th);
-    for (auto& t : pool) t.join();
-  }
-  for (int th = 0; th < nth; th++)
-    if (fail[th]) {
-      dst->err = "transfer: a new cell lies in no old cell";
-      return NRD_EINVAL;
-    }
-  size_t nrec = 0;
-  for (const auto& v : recs) nrec += v.size();
-  std::vector<ReconDesc> rec;
-  rec.reserve(nrec);
-  for (const auto& v : recs) rec.insert(rec.end(), v.begin(), v.end());
-  const size_t No = (size_t)A.N, Nn = (size_t)B.N;
-  // one device buffer: the old vectors (made composite), the codes and the
-  // reconstruction entries
-  const size_t comp_bytes = 2 * No * nvec * sizeof(double);
-  const size_t code_bytes = (Nn * sizeof(int) + 15) / 16 * 16;
-  const size_t rec_bytes = nrec * sizeof(ReconDesc);
-  char* d_buf = nullptr;
-  if (cudaMalloc(&d_buf, comp_bytes + code_bytes + rec_bytes) != cudaSuccess) {
+  const size_t No = (size_t)A.N;
+  // composite copies of the old vectors (with finer levels) and the covered
+  // slots of the level below the finest, in a buffer the old context keeps
+  const bool comp = A.L > 1;
+  const size_t comp_bytes = comp ? 2 * No * nvec * sizeof(double) : 0;
+  const size_t slot_bytes = comp ? (size_t)A.lev[A.L - 2].ncell * sizeof(int) : 0;
+  if (comp && !xfer_reserve(src, comp_bytes + slot_bytes)) {
     dst->err = "allocation failed";
     return NRD_ENOMEM;
   }
-  double* d_comp = (double*)d_buf;
-  int* d_code = (int*)(d_buf + comp_bytes);
-  ReconDesc* d_rec = (ReconDesc*)(d_buf + comp_bytes + code_bytes);
-  cudaMemcpyAsync(d_code, code.data(), Nn * sizeof(int), cudaMemcpyHostToDevice, s);
-  if (nrec) cudaMemcpyAsync(d_rec, rec.data(), rec_bytes, cudaMemcpyHostToDevice, s);
+  OldCells O{};
+  O.L = A.L;
+  for (int l = 0; l < A.L; l++) {
+    for (int d = 0; d < 3; d++) O.n[l][d] = A.lev[l].n[d];
+    O.lmap[l] = A.d_lmap[l];
+  }
+  const double* old = u_src;
   dst->timer.begin(NRD_TK_TRANSFER, s);
-  cudaMemcpyAsync(d_comp, u_src, comp_bytes, cudaMemcpyDeviceToDevice, s);
-  launch_average_down(A, d_comp, 2 * nvec, (int)No, s);
-  const long work_items = (long)Nn + (long)nrec;
-  const int grid = (int)std::max(1L, std::min(152L * 8, (work_items + 255) / 256));
-  k_transfer<<<grid, 256, 0, s>>>(d_code, d_rec, (int)Nn, (int)nrec, (int)No, nvec, d_comp,
-                                  u_dst);
+  if (comp) {
+    const int lp = A.L - 2;
+    double* d_comp = (double*)src->d_xfer;
+    int* slot = (int*)((char*)src->d_xfer + comp_bytes);
+    cudaMemcpyAsync(d_comp, u_src, comp_bytes, cudaMemcpyDeviceToDevice, s);
+    launch_average_down(A, d_comp, 2 * nvec, (int)No, s);
+    cudaMemsetAsync(slot, 0xff, slot_bytes, s);
+    if (A.ncov[lp])
+      k_cov_slots<<<rg_blocks(A.ncov[lp]), 256, 0, s>>>(A.d_cov[lp], A.ncov[lp], A.lev[lp].off,
+                                                        slot);
+    O.cov = A.d_cov[lp];
+    O.slot = slot;
+    O.off = A.lev[lp].off;
+    old = d_comp;
+  }
+  k_transfer<<<(int)B.tiles.size(), 256, 0, s>>>(B.d_tiles, B.d_patches, B.tile_x, B.tile_y, O,
+                                                 B.N, (int)No, nvec, old, u_dst);
   dst->timer.end(NRD_TK_TRANSFER, s);
   const cudaError_t e = cudaStreamSynchronize(s);
-  cudaFree(d_buf);
+  xfer_done(src);
   if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) {
     dst->err = "transfer kernel failed";
     return NRD_ECUDA;

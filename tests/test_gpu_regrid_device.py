@@ -1,0 +1,73 @@
+"""The device side of clustering and transfer at its edges, against the
+oracle: row lengths around the 32-cell scans, buffers wider than a box side,
+new hierarchies shallower, as deep as and deeper than the old one (finest
+cells found through the covered list, or through the box of a single level),
+several vectors, repeated calls with growing scratch.  Boxes are integers and
+must be equal; the transfer's bound is that of the other transfer tests,
+1e-14 of max |u| (two FP64 operations per axis)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+from oracle import regrid as R  # noqa: E402
+from paper_1302_6303_gb300 import workloads as W  # noqa: E402
+from regrid_cases import random_hierarchy  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def nrd():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+    from paper_1302_6303_gb300 import nrd as m
+    return m
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def ctx_for(nrd, h):
+    ctx = nrd.Context(nmg=1)
+    ctx.set_hierarchy_from(h)
+    ctx.set_material(dev(np.ones(h.ncells, np.float32)))
+    return ctx
+
+
+def as_lists(levels):
+    return [[(tuple(lo), tuple(hi)) for lo, hi in lev] for lev in levels]
+
+
+@pytest.mark.parametrize("n0", [(33, 5, 4), (31, 7, 3), (32, 4, 6), (1, 9, 8), (65, 3, 3)])
+@pytest.mark.parametrize("levels", [1, 2])
+def test_boxes(nrd, n0, levels):
+    rng = np.random.default_rng(sum(n0) + levels)
+    h = W.uniform(n0) if levels == 1 else random_hierarchy(rng, n0, 2, count=2, side_lo=2,
+                                                           side_hi=4)
+    tags = (rng.random(h.ncells) < 0.08).astype(np.uint8) * 2
+    ctx = ctx_for(nrd, h)
+    for buf, eff, mn, mx, ml in [(0, 0.6, 2, 8, 2), (1, 0.7, 2, 32, 3), (6, 0.7, 4, 16, 3)]:
+        got = ctx.regrid_boxes(dev(tags), 2, buf, eff, mn, mx, ml)
+        exp = R.regrid_boxes(h, tags, tag_bits=2, buffer=buf, efficiency=eff, min_side=mn,
+                             max_side=mx, max_levels=ml)
+        assert as_lists(got) == as_lists(exp)
+
+
+@pytest.mark.parametrize("old", [1, 2, 3])
+@pytest.mark.parametrize("new", [1, 2, 3])
+def test_transfer_depths(nrd, old, new):
+    rng = np.random.default_rng(10 * old + new)
+    n0 = (9, 6, 7)
+    mk = lambda L: W.uniform(n0) if L == 1 else random_hierarchy(rng, n0, L)  # noqa: E731
+    a, b = mk(old), mk(new)
+    ca, cb = ctx_for(nrd, a), ctx_for(nrd, b)
+    for nvec in (1, 3):
+        u = rng.uniform(0.1, 2.0, (nvec, 2 * a.ncells))
+        out = ca.transfer_to(cb, dev(u)).cpu().numpy()
+        for v, o in zip(u, out):
+            exp = R.transfer(a, b, v)
+            assert np.abs(o - exp).max() <= 1e-14 * np.abs(exp).max()
