@@ -9,6 +9,7 @@
 #include <utility>
 
 #include "nrd_internal.h"
+#include "softfp.h"
 
 namespace {
 
@@ -641,8 +642,10 @@ __device__ __forceinline__ void orth_final_n(const double* __restrict__ w, doubl
     double wE = w[i], wT = w[N + i];
     if (NV > 0) sub_cols<(NV > 0 ? NV : 1)>(wE, wT, V, stride, i, N, h);
     else sub_all(wE, wT, V, stride, i, N, nv, h);
-    vn[i] = sc * wE;
-    vn[N + i] = sc * wT;
+    // the scaling on the integer pipe (the same bits; a quarter to an eighth of
+    // the sweep's FP64 instructions in the usual short bases)
+    vn[i] = soft_mul_any(sc, wE);
+    vn[N + i] = soft_mul_any(sc, wT);
   }
 }
 __device__ __forceinline__ void orth_final(const double* w, double* V, long stride, int N, int nv,
