@@ -538,13 +538,12 @@ static int step_prepare(nrd_ctx* c, double* u, const double* u_n, const double* 
   rc = solver_alloc(c);
   if (rc != NRD_OK) return rc;
   const int n2 = 2 * c->H.N;
-  cudaMemcpyAsync(c->d_b, u_n, n2 * sizeof(double), cudaMemcpyDeviceToDevice, s);
   if (u_nm1) {
     const double al = dt / dt_prev;
     *a0 = (1.0 + 2.0 * al) / (1.0 + al);
-    launch_axpy(n2, al, u_n, c->d_b, s);                       // (1 + al) u_n
-    launch_axpy(n2, -al * al / (1.0 + al), u_nm1, c->d_b, s);
+    launch_history(n2, al, -al * al / (1.0 + al), u_n, u_nm1, c->d_b, s);
   } else {
+    cudaMemcpyAsync(c->d_b, u_n, n2 * sizeof(double), cudaMemcpyDeviceToDevice, s);
     *a0 = 1.0;
   }
   return NRD_OK;
@@ -581,12 +580,18 @@ int nrd_tag(nrd_ctx* c, const double* u, double thr_c, double thr_g, double thr_
   if (!u || !tags) return fail(c, NRD_EINVAL, "null argument");
   Hier& H = c->H;
   size_t N = H.N;
-  // composite values: covered cells := mean of their children
-  cudaMemcpyAsync(c->d_tmp, u, 2 * N * sizeof(double), cudaMemcpyDeviceToDevice, s);
-  launch_average_down(H, c->d_tmp, 2, (int)N, s);
-  launch_ghost_fill(H, c->mp, c->d_z, c->d_tmp, c->d_gu, 1, s);
-  launch_emax(H, c->R, u, 2, s);
-  launch_tag(H, c->d_tmp, c->d_gu, thr_c, thr_g, thr_r, c->R.d_res + 2, tags, s);
+  // composite values: covered cells := mean of their children (one level has
+  // none: its own values)
+  const double* uc = u;
+  if (H.L > 1) {
+    cudaMemcpyAsync(c->d_tmp, u, 2 * N * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    launch_average_down(H, c->d_tmp, 2, (int)N, s);
+    uc = c->d_tmp;
+  }
+  launch_ghost_fill(H, c->mp, c->d_z, uc, c->d_gu, 1, s);
+  // max |E| scales tau^c and tau^g only (an infinite threshold never tags)
+  if (!(thr_c == INFINITY && thr_g == INFINITY)) launch_emax(H, c->R, u, 2, s);
+  launch_tag(H, uc, c->d_gu, thr_c, thr_g, thr_r, c->R.d_res + 2, tags, s);
   return check_launch(c);
 }
 

@@ -211,6 +211,9 @@ void launch_emax(const Hier& H, Reducer& R, const double* E, int slot, cudaStrea
 // multi-dot: res[slot + i] = <w, V_i> for i < nv (V given as base + i*stride)
 // w -= sum_i h[i] V_i  (h device)
 void launch_axpy(int n, double a, const double* x, double* y, cudaStream_t s);
+// b = (1 + al) x + c2 y (the history combination of Eq. bdf2), as x + al x + c2 y
+void launch_history(int n, double al, double c2, const double* x, const double* y, double* b,
+                    cudaStream_t s);
 void launch_scale_dev(int n, const double* num, const double* den_sq, double* x, cudaStream_t s);
 void launch_lincomb_dev(int n, double* x, const double* Z, long stride, int nv, const double* y,
                         cudaStream_t s);
