@@ -104,42 +104,45 @@ WORKLOADS = {
 #    P1 coefficients 2: 31 ops and 2 divisions (1/T_f, 1/(E_a + E_b)); per
 #    cell the coupling partials 7 ops and 1 division, the P2 data 4 ops and
 #    1 division: 194 ops, 18 divisions, 3 square roots.
-#  frozen Jv: per face 6 + 3 (the two tangent fluxes from the five partials),
-#    per cell the two divergences 16, the coupling tangent 3, a0 v - dt (...)
-#    6: 52 ops.
+#    (The sums of a cell's own Jacobian entries, which the frozen Jv then need
+#    not form, are not counted.)
+#  frozen Jv, one sum per row: the two own entries 3 + 3, six neighbours with
+#    two products in the E row and one in the T row 36, a0 v - dt (...) 6: 48 ops.
 LIN_OPS = (194, 18, 3)            # (ops, divisions, square roots) per leaf cell
 RES_OPS = (90, 10, 3)
-JV_OPS = (52, 0, 0)
-# frozen-Jacobian Jv: 3 faces x 5 partials x 8 B + v 16 B + cell partials
-# 16 B + Jv 16 B + mask 1 B
-JV_BYTES_PER_CELL = 169.0
+JV_OPS = (48, 0, 0)
+# frozen-Jacobian Jv: 3 faces x 5 partials x 8 B + own entries 32 B + v 16 B
+# + Jv 16 B + mask 1 B
+JV_BYTES_PER_CELL = 185.0
 # DRAM bytes per launch group from an ncu capture of the current kernels,
 # per workload (None: not captured for this kernel version and workload)
 # (single256: captured on the same layout at 128^3, 2,097,152 cells, and
 # scaled by the cells, x8: these stencils stream their inputs once; the
-# linearisation's face and cell launches 58.1 + 394.5 + 187.8 + 64.9 MB,
-# the frozen Jv 322.0 + 55.6 MB)
+# linearisation's face and cell launches 58.0 + 400.0 + 441.9 + 129.1 MB,
+# the frozen Jv 356.0 + 46.9 MB)
 TRAFFIC = {
     "amr2_base64": {"linearise": None, "jv": None},
     "batching_base128": {"linearise": None, "jv": None},
-    "single256": {"linearise": 8 * (58.1 + 394.5 + 187.8 + 64.9) * 1e6,
-                  "jv": 8 * (322.0 + 55.6) * 1e6},
+    "single256": {"linearise": 8 * (58.0 + 400.0 + 441.9 + 129.1) * 1e6,
+                  "jv": 8 * (356.0 + 46.9) * 1e6},
 }
 # FP64-pipe instructions per cell measured by ncu (sm__inst_executed_pipe_fp64,
-# same capture): linearisation 139.2 + 35.0, frozen Jv 40.4
-LIN_INST_NCU, JV_INST_NCU = 139.2 + 35.0, 40.4
+# same capture): linearisation 67.1 + 40.0, frozen Jv 24.6 (about half the
+# products run on the integer pipe and are not in these counts)
+LIN_INST_NCU, JV_INST_NCU = 67.1 + 40.0, 24.6
 # Algorithmic DRAM bytes per leaf cell of the linearisation as laid out here:
 # face launch reads E, T, z^3 (24 B) and writes per face slot (3 per cell) the
 # 5 FP64 Jacobian partials, the 2 scaled FP32 P1 coefficients and the 2 FP64
-# face fluxes (3 x 64 = 192 B); the cell launch reads the 6 fluxes of its
-# low faces (48 B), u and b (32 B) and z^3 (8 B) and writes F (16 B), the 2
-# FP64 coupling partials (16 B) and the 3 FP32 P2 values (12 B).  The residual
+# face fluxes (3 x 64 = 192 B); the cell launch reads the 6 fluxes (48 B) and
+# the 15 partials (120 B) of its low faces, u and b (32 B) and z^3 (8 B) and
+# writes F (16 B), its 4 FP64 own Jacobian entries (32 B) and the 3 FP32 P2
+# values (12 B).  The residual
 # alone moves 52 B per cell and the analytic Jv 52 B (E, T, v, z read, Jv
 # written); the frozen form stores the partials once per Newton iterate so
 # that each Krylov iteration reads them instead of recomputing them in FP64.
 # (ncu's DRAM bytes of a launch can fall below these counts: writes still held
 # in the 129 MB L2 when the launch ends are counted by a later one.)
-LIN_BYTES_PER_CELL = 24 + 192 + 48 + 32 + 8 + 16 + 16 + 12
+LIN_BYTES_PER_CELL = 24 + 192 + 48 + 120 + 32 + 8 + 16 + 32 + 12
 RES_BYTES_PER_CELL = 52.0
 
 
@@ -924,7 +927,7 @@ def main():
                          "residual_only_per_cell": RES_BYTES_PER_CELL,
                          "ratio_to_residual_only": tpc / RES_BYTES_PER_CELL,
                          "why": "the linearisation also writes the frozen Jacobian partials, "
-                                "P1 coefficients, coupling partials and P2 data that the "
+                                "own entries, P1 coefficients and P2 data that the "
                                 "Krylov iterations and the V-cycle read (FP64 issue, not "
                                 "HBM, bounds these kernels)"}
     jv_ms, jv_n = kt["jv"]
@@ -932,7 +935,7 @@ def main():
     ach_jv = flops(JV_OPS) * leaf / t_jv / 1e9
     ach_jv_inst = JV_INST_NCU * leaf / t_jv / 1e9
     gbs_jv = JV_BYTES_PER_CELL * leaf / t_jv / 1e9
-    roof_jv = {"kernel": "k_stencil<ST_JVF> (frozen-Jacobian Jv)", "bound": "alu",
+    roof_jv = {"kernel": "k_jv_frozen (frozen-Jacobian Jv, row sums)", "bound": "alu",
                "achieved": ach_jv, "peak": flop_peak, "unit": "GFLOP/s (FP64)",
                "frac": ach_jv / flop_peak, "traffic": traffic.get("jv"),
                "per_launch_us": t_jv * 1e6, "launches": jv_n,
@@ -949,9 +952,10 @@ def main():
                             "ratio": tpc / JV_BYTES_PER_CELL,
                             "analytic_jv_per_cell": RES_BYTES_PER_CELL,
                             "ratio_to_analytic": tpc / RES_BYTES_PER_CELL,
-                            "why": "reads the 5 stored FP64 partials per face instead of "
-                                   "re-deriving them from E, T and z (40 FP64 instructions "
-                                   "per cell instead of about 130)"}
+                            "why": "reads the 5 stored FP64 partials per face and 4 own "
+                                   "entries per cell instead of re-deriving them from E, T "
+                                   "and z (25 FP64 instructions per cell instead of about "
+                                   "130)"}
     pc_ms, pc_n = kt["pc_apply"]
     t_pc = pc_ms / max(pc_n, 1) * 1e-3
     vb = vcycle_bytes_per_cell(h, sweeps)

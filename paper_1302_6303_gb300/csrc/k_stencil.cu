@@ -2,8 +2,10 @@
 // and its Jacobian-vector products (Sec. 4.1), all FP64:
 //   ghost fill     physical / sibling / coarse-fine ghosts from a work-list
 //   k_stencil      one persistent launch over the tiles of every level:
-//                  halo staged in shared memory, each face flux computed
-//                  once and shared by its two cells, then the cell balance
+//                  halo staged in shared memory; the residual and the
+//                  linearisation as a face launch (each face once) and a
+//                  cell launch, the exact and FD Jv in one
+//   k_jv_frozen    the frozen Jacobian's product, one row sum per cell and field
 //   k_reflux       flux matching at coarse-fine faces
 //   k_tag          Sec. 5 refinement indicators
 //   k_avgdown      covered cells := mean of their children
@@ -858,14 +860,14 @@ struct JvArgs {
   const double* par;
 };
 
-// Frozen Jv: out = a0 v - dt L v, one row sum per cell and field (26 FP64
-// instructions) over the 19 coefficients of the cell; fine-side coarse-fine
+// Frozen Jv: out = a0 v - dt L v, one row sum per cell and field (24.6 FP64
+// instructions, counted) over the 19 coefficients of the cell; fine-side coarse-fine
 // fluxes to cf for flux matching.  One tile of the stencil list per block.
 // In flux form (each face's two tangent fluxes, then the divergence) a cell
 // took 40 FP64 instructions and the kernel was bound by the FP64 pipe; the
 // rows move 9% more bytes.  Its four plain products run on the integer pipe.
-// At 256^3: 1.30 -> 0.70 ms (six blocks per SM; the compiler's own choice of
-// three 0.76), 0.69 of the FP64 issue rate being the bound left.
+// At 256^3: 1.30 -> 0.69 ms (six blocks per SM; the compiler's own choice of
+// three 0.76): 0.95 of the FP64 issue rate, the bound left, and 0.69 of HBM.
 __global__ void __launch_bounds__(256, 6) k_jv_frozen(JvArgs A) {
   const int N = A.N, G = A.G;
   double a0 = A.a0, dt = A.dt;

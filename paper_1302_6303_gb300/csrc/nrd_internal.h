@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -334,7 +335,10 @@ struct nrd_ctx {
   double* d_gv = nullptr;      // 2G: ghosts of a direction
   double* d_cf = nullptr;      // 2G: fine-side coarse-fine fluxes
   double* d_tmp = nullptr;     // 2N scratch
-  void* d_xfer = nullptr;      // scratch of nrd_regrid_boxes and nrd_transfer (regrid.cu)
+  // scratch of nrd_regrid_boxes and nrd_transfer (regrid.cu); a call holds the
+  // mutex while it uses it (several threads may transfer from one context)
+  std::mutex xfer_mu;
+  void* d_xfer = nullptr;
   size_t xfer_bytes = 0;
   Jac jac;                     // frozen Jacobian (one allocation, at jac.jc)
   double* d_pef = nullptr;     // [2][3N+G] face fluxes of the split linearisation

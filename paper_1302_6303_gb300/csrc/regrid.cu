@@ -394,7 +394,9 @@ void xfer_done(nrd_ctx* c) {
 // the device fields and tables of one level
 struct RgDevice {
   nrd_ctx* c;
-  ~RgDevice() { xfer_done(c); }
+  std::lock_guard<std::mutex> lock;
+  explicit RgDevice(nrd_ctx* ctx) : c(ctx), lock(ctx->xfer_mu) {}
+  ~RgDevice() { xfer_done(c); }   // before the lock is released
   // tables of the tagged cells and (unless the level covers the domain) of the
   // nestable cells, on the host; false when the device had no memory for it
   bool tables(const Hier& H, const uint8_t* tags, int bits, int buffer, int l, const int n[3],
@@ -681,6 +683,8 @@ int nrd_transfer(nrd_ctx* src, nrd_ctx* dst, const double* u_src, double* u_dst,
   const bool comp = A.L > 1;
   const size_t comp_bytes = comp ? 2 * No * nvec * sizeof(double) : 0;
   const size_t slot_bytes = comp ? (size_t)A.lev[A.L - 2].ncell * sizeof(int) : 0;
+  std::unique_lock<std::mutex> lock(src->xfer_mu, std::defer_lock);
+  if (comp) lock.lock();   // until the call returns: its kernels have ended then
   if (comp && !xfer_reserve(src, comp_bytes + slot_bytes)) {
     dst->err = "allocation failed";
     return NRD_ENOMEM;
@@ -712,7 +716,7 @@ int nrd_transfer(nrd_ctx* src, nrd_ctx* dst, const double* u_src, double* u_dst,
                                                  B.N, (int)No, nvec, old, u_dst);
   dst->timer.end(NRD_TK_TRANSFER, s);
   const cudaError_t e = cudaStreamSynchronize(s);
-  xfer_done(src);
+  if (comp) xfer_done(src);
   if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) {
     dst->err = "transfer kernel failed";
     return NRD_ECUDA;

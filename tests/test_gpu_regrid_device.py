@@ -5,6 +5,8 @@ cells found through the covered list, or through the box of a single level),
 several vectors, repeated calls with growing scratch.  Boxes are integers and
 must be equal; the transfer's bound is that of the other transfer tests,
 1e-14 of max |u| (two FP64 operations per axis)."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -71,3 +73,32 @@ def test_transfer_depths(nrd, old, new):
         for v, o in zip(u, out):
             exp = R.transfer(a, b, v)
             assert np.abs(o - exp).max() <= 1e-14 * np.abs(exp).max()
+
+
+def test_transfer_threads(nrd):
+    """Two threads, each with a stream and a destination of its own, transfer
+    from one context whose scratch they share; the values are those of the
+    same calls one after the other."""
+    rng = np.random.default_rng(5)
+    n0 = (17, 12, 9)
+    a, b = random_hierarchy(rng, n0, 2), random_hierarchy(rng, n0, 3)
+    ca = ctx_for(nrd, a)
+    cb = [ctx_for(nrd, b), ctx_for(nrd, b)]
+    us = [[dev(rng.uniform(0.1, 2.0, (nv, 2 * a.ncells))) for nv in (1, 4, 2, 6)] for _ in cb]
+    exp = [[ca.transfer_to(c, u) for u in w] for c, w in zip(cb, us)]
+    torch.cuda.synchronize()
+    got = [[], []]
+
+    def work(t):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(5):
+                got[t] = [ca.transfer_to(cb[t], u) for u in us[t]]
+
+    th = [threading.Thread(target=work, args=(t,)) for t in range(2)]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    torch.cuda.synchronize()
+    for g, e in zip(got, exp):
+        assert len(g) == len(e) and all(torch.equal(x, y) for x, y in zip(g, e))
