@@ -10,6 +10,7 @@
 //   k_tag          Sec. 5 refinement indicators
 //   k_avgdown      covered cells := mean of their children
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <type_traits>
 
@@ -26,11 +27,8 @@ struct LevelH {
   // constants of face_core
   double c1[NRD_MAX_LEVELS][3];   // 1 / (12 h^2)
   double cLh[NRD_MAX_LEVELS][3];  // (cL / 2) h
-  double cT[NRD_MAX_LEVELS][3];   // 2^(-5/2) k / h^2
+  double cT[NRD_MAX_LEVELS][3];   // 2^(-5/2) k / h^2 (Tf^(5/2) = 2^(-5/2) Ts^(5/2), Ts = T_a + T_b)
 };
-
-// 2^(-5/2): Tf^(5/2) = 2^(-5/2) Ts^(5/2) with Ts = T_a + T_b
-constexpr double kP52 = 0.17677669529663688;
 
 struct GhostArgs {
   const uint8_t* gtype;
@@ -866,8 +864,10 @@ struct JvArgs {
 // In flux form (each face's two tangent fluxes, then the divergence) a cell
 // took 40 FP64 instructions and the kernel was bound by the FP64 pipe; the
 // rows move 9% more bytes.  Its four plain products run on the integer pipe.
-// At 256^3: 1.30 -> 0.69 ms (six blocks per SM; the compiler's own choice of
-// three 0.76): 0.95 of the FP64 issue rate, the bound left, and 0.69 of HBM.
+// At 256^3: 1.30 -> 0.73 ms (six blocks per SM; with five 0.78): 0.90 of the
+// FP64 issue rate, the bound left, and 0.63 of HBM.  The row's order costs
+// 0.04 ms against own entries first, whose rounding error is a fifth larger
+// (2.5e-16 in the 2-norm against 2.1e-16 here, 2.2e-16 in flux form).
 __global__ void __launch_bounds__(256, 6) k_jv_frozen(JvArgs A) {
   const int N = A.N, G = A.G;
   double a0 = A.a0, dt = A.dt;
@@ -896,9 +896,10 @@ __global__ void __launch_bounds__(256, 6) k_jv_frozen(JvArgs A) {
     const double* vE = A.v;
     const double* vT = A.v + N;
     const double vEc = vE[idx], vTc = vT[idx];
-    // the four plain products on the integer pipe (bit-identical)
-    double LE = fma(J.cen[N + idx], vTc, soft_mul_any(J.cen[idx], vEc));
-    double LT = fma(J.cen[3L * N + idx], vEc, soft_mul_any(J.cen[2L * N + idx], vTc));
+    // A row's largest terms (the diagonal; in the T row the coupling too) come
+    // last: fewer of its roundings are then of its full size.  The plain
+    // products run on the integer pipe (bit-identical).
+    double LE = soft_mul_any(J.cen[N + idx], vTc), LT = 0.0;
     const bool inner = i > 0 && i < nx - 1 && j > 0 && j < ny - 1 && k > 0 && k < nz - 1;
     const long NS = 3L * N + G;
     if (inner && m == 0) {
@@ -911,7 +912,7 @@ __global__ void __launch_bounds__(256, 6) k_jv_frozen(JvArgs A) {
         const double tl = vT[lo], th = vT[hi];
         LE = fma(-jl[0], vE[lo], LE);
         LE = fma(-jl[2 * NS], tl, LE);
-        LT = fma(-jl[3 * NS], tl, LT);
+        LT = d ? fma(-jl[3 * NS], tl, LT) : soft_mul_any(-jl[3 * NS], tl);
         LE = fma(jh[NS], vE[hi], LE);
         LE = fma(jh[2 * NS], th, LE);
         LT = fma(jh[4 * NS], th, LT);
@@ -951,6 +952,9 @@ __global__ void __launch_bounds__(256, 6) k_jv_frozen(JvArgs A) {
         }
       }
     }
+    LE = fma(J.cen[idx], vEc, LE);
+    LT = fma(J.cen[3L * N + idx], vEc, LT);
+    LT = fma(J.cen[2L * N + idx], vTc, LT);
     A.out[idx] = fma(-dt, LE, soft_mul_any(a0, vEc));
     A.out[N + idx] = fma(-dt, LT, soft_mul_any(a0, vTc));
   }
@@ -1156,9 +1160,11 @@ LevelH level_h(const Hier& H, double k = 0.01, double cL = 4.0) {
       lh.rh[l][d] = 1.0 / h;
       lh.h3[l][d] = 3.0 * h;
       lh.kh[l][d] = k / h;
-      lh.c1[l][d] = 1.0 / (12.0 * h * h);
-      lh.cLh[l][d] = 0.5 * cL * h;
-      lh.cT[l][d] = kP52 * (k / (h * h));
+      // from the level's extent n = 1/h, one rounding each
+      const long double n = (l < H.L) ? H.lev[l].n[d] : 1;
+      lh.c1[l][d] = (double)(n * n / 12.0L);
+      lh.cLh[l][d] = (double)(0.5L * cL / n);
+      lh.cT[l][d] = (double)(std::sqrt(0.03125L) * k * (n * n));
     }
   return lh;
 }

@@ -104,9 +104,10 @@ __global__ void __launch_bounds__(256, 6) k_vjp_cells(VjpArgs a) {
       continue;
     }
     const double wEc = wE[idx], wTc = wT[idx];
-    // the four plain products on the integer pipe (bit-identical)
-    double aE = fma(J.cen[3L * N + idx], wTc, soft_mul_any(J.cen[idx], wEc));
-    double aT = fma(J.cen[N + idx], wEc, soft_mul_any(J.cen[2L * N + idx], wTc));
+    // the four plain products on the integer pipe (bit-identical); the diagonal
+    // last, as in the product
+    double aE = soft_mul_any(J.cen[3L * N + idx], wTc);
+    double aT = soft_mul_any(J.cen[N + idx], wEc);
     double aZ = 0.0;
     const int pos[3] = {i, j, k};
 #pragma unroll
@@ -146,6 +147,8 @@ __global__ void __launch_bounds__(256, 6) k_vjp_cells(VjpArgs a) {
       aE += wq * a.gam[g];
       aT += wq * a.gam[G + g];
     }
+    aE = fma(J.cen[idx], wEc, aE);
+    aT = fma(J.cen[2L * N + idx], wTc, aT);
     a.out[idx] = fma(-a.dt, aE, soft_mul_any(a.a0, wEc));
     a.out[N + idx] = fma(-a.dt, aT, soft_mul_any(a.a0, wTc));
     if (DZ) {
