@@ -319,7 +319,9 @@ int nrd_tag(nrd_ctx* ctx, const double* u, double thr_c, double thr_g, double th
  * signatures, else in the middle of its longest side, each part keeping at
  * least min_side/2 planes unless proper nesting forces a narrower cut.  The
  * accepted boxes refined by 2 form level l+1.
- *   tags: device, ncells bytes (nrd_tag's output);  min_side, max_side: even,
+ *   tags: device, ncells bytes: the output of the last nrd_tag on this context,
+ *   on any stream (the call waits for it; a captured nrd_tag does not count), or
+ *   bytes that the legacy default stream may read;  min_side, max_side: even,
  *   2 <= min_side <= max_side, in cells of the new level;  max_levels: 1 ..
  *   NRD_MAX_LEVELS, levels of the new hierarchy at most;  out (host):
  *   *nlevels_out levels, nboxes_out[max_levels] boxes per level (0 past the
@@ -328,7 +330,8 @@ int nrd_tag(nrd_ctx* ctx, const double* u, double thr_c, double thr_g, double th
  *   it exceeds max_boxes, which returns NRD_EINVAL, as does a level whose
  *   index space has 2^31 cells or more).  The fields of a level (about 14 bytes
  *   per cell of its index space) are formed in device memory, on the host when
- *   that is not to be had.  Synchronises. */
+ *   that is not to be had.  Works on the legacy default stream and
+ *   synchronises. */
 int nrd_regrid_boxes(nrd_ctx* ctx, const uint8_t* tags, int tag_bits, int buffer,
                      double efficiency, int min_side, int max_side, int max_levels,
                      int max_boxes, int* nlevels_out, int* nboxes_out, int* boxes_out,

@@ -264,6 +264,7 @@ int nrd_destroy(nrd_ctx* c) {
   if (!c) return NRD_EINVAL;
   if (c->pend) cudaStreamSynchronize(c->pend_s);   // nothing in flight may outlive the buffers
   c->timer.destroy();
+  if (c->tag_ev) cudaEventDestroy(c->tag_ev);
   free_fields(c);
   if (c->have_hier) hier_free(c->H);
   delete c;
@@ -592,6 +593,17 @@ int nrd_tag(nrd_ctx* c, const double* u, double thr_c, double thr_g, double thr_
   // max |E| scales tau^c and tau^g only (an infinite threshold never tags)
   if (!(thr_c == INFINITY && thr_g == INFINITY)) launch_emax(H, c->R, u, 2, s);
   launch_tag(H, uc, c->d_gu, thr_c, thr_g, thr_r, c->R.d_res + 2, tags, s);
+  // the clustering has no stream argument and runs on the legacy default one: an
+  // event orders it after tags from another (not from inside a capture, whose
+  // events are not for use outside it)
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (s && s != cudaStreamLegacy &&
+      !(cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)) {
+    if ((!c->tag_ev &&
+         cudaEventCreateWithFlags(&c->tag_ev, cudaEventDisableTiming) != cudaSuccess) ||
+        cudaEventRecord(c->tag_ev, s) != cudaSuccess)
+      return fail(c, NRD_ECUDA, "event after the tags failed");
+  }
   return check_launch(c);
 }
 

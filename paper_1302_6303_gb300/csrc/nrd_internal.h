@@ -335,6 +335,9 @@ struct nrd_ctx {
   double* d_gv = nullptr;      // 2G: ghosts of a direction
   double* d_cf = nullptr;      // 2G: fine-side coarse-fine fluxes
   double* d_tmp = nullptr;     // 2N scratch
+  // the end of the last nrd_tag on a stream of its own; the clustering, which
+  // runs on the legacy default stream, waits for it
+  cudaEvent_t tag_ev = nullptr;
   // scratch of nrd_regrid_boxes and nrd_transfer (regrid.cu); a call holds the
   // mutex while it uses it (several threads may transfer from one context)
   std::mutex xfer_mu;

@@ -552,6 +552,11 @@ int nrd_regrid_boxes(nrd_ctx* c, const uint8_t* tags, int tag_bits, int buffer,
     c->err = "bad argument to nrd_regrid_boxes";
     return NRD_EINVAL;
   }
+  // the work below goes to the legacy default stream, after the tags
+  if (c->tag_ev && cudaStreamWaitEvent(nullptr, c->tag_ev, 0) != cudaSuccess) {
+    c->err = "wait for the tags failed";
+    return NRD_ECUDA;
+  }
   const Hier& H = c->H;
   std::vector<uint8_t> htags;   // filled when a level is done on the host
   const int n0[3] = {H.lev[0].n[0], H.lev[0].n[1], H.lev[0].n[2]};

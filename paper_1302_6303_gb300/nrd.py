@@ -449,6 +449,11 @@ class Context:
         (nrd_regrid_boxes); returns levels[l] = [(lo, hi), ...]."""
         if max_levels is None:
             max_levels = self.nlevels
+        # the call works on the legacy default stream: tags written on another
+        # current stream (by nrd_tag or by torch) are waited for here
+        s = torch.cuda.current_stream()
+        if s.cuda_stream:
+            s.synchronize()
         nl, tot = ctypes.c_int(), ctypes.c_int()
         nb = (ctypes.c_int * max_levels)()
         bx = (ctypes.c_int * (6 * max_boxes))()

@@ -102,3 +102,35 @@ def test_transfer_threads(nrd):
     torch.cuda.synchronize()
     for g, e in zip(got, exp):
         assert len(g) == len(e) and all(torch.equal(x, y) for x, y in zip(g, e))
+
+
+@pytest.mark.parametrize("cluster", ["tag side", "tag default", "copy side"])
+def test_tags_from_another_stream(nrd, cluster):
+    """Tags written late on a side stream, by nrd_tag or by torch, are the ones
+    clustered, from that stream or (nrd_tag's) from the default one: the boxes
+    are those of the same tags made and clustered on the default stream."""
+    h = W.uniform(24)
+    u = dev(W.front_state(h, seed=4, noise=0.0, front=0.4, width=0.1))
+    ctx = ctx_for(nrd, h)
+    ref = ctx.tag(u, thr_r=0.1)
+    boxes = lambda t: as_lists(ctx.regrid_boxes(t, 4, 1, 0.7, 4, 16, 2))  # noqa: E731
+    exp = boxes(ref)
+    assert len(exp) == 2
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        for _ in range(2):   # (untagged bytes are what an early read would find)
+            torch.zeros(h.ncells, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        if cluster == "copy side":
+            tags = torch.zeros_like(ref)
+            torch.cuda._sleep(200_000_000)
+            tags.copy_(ref)
+        else:
+            torch.cuda._sleep(200_000_000)
+            tags = ctx.tag(u, thr_r=0.1)
+        if cluster != "tag default":
+            got = boxes(tags)
+    if cluster == "tag default":
+        got = boxes(tags)
+    assert got == exp
