@@ -31,7 +31,9 @@
  *     through host pointers).
  *   - The context owns its internal device work buffers (allocated in
  *     nrd_set_hierarchy and on first use by the solver calls) and frees them
- *     in nrd_destroy.  A context is used by one host thread at a time.
+ *     in nrd_destroy.  A context is used by one host thread at a time, except
+ *     as the source of nrd_transfer: several threads may transfer from one
+ *     context at once, each on a stream and to a context of its own.
  *
  * Data layout (the "hierarchy layout")
  *   - A hierarchy has L levels; level 0 is one box [0,n0x) x [0,n0y) x
@@ -350,7 +352,8 @@ int nrd_regrid_boxes(nrd_ctx* ctx, const uint8_t* tags, int tag_bits, int buffer
  *   nvec x 2*ncells(dst) doubles (every cell written).  Where the old
  * hierarchy has finer levels, ctx_src holds a device buffer for it: a copy of
  * u_src and 4 bytes per cell of the level below the finest (kept up to 256 MB,
- * else freed before the call returns).  Synchronises.
+ * else freed before the call returns; a call that finds it in use by another
+ * thread's allocates its own for the call).  Synchronises the stream.
  * Errors: NRD_ESTATE (a context without hierarchy), NRD_EINVAL (different
  * base grids, null pointers, nvec < 1),
  * NRD_ENOMEM, NRD_ECUDA; the message is stored in ctx_dst. */

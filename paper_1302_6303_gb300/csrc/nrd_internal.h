@@ -339,7 +339,8 @@ struct nrd_ctx {
   // runs on the legacy default stream, waits for it
   cudaEvent_t tag_ev = nullptr;
   // scratch of nrd_regrid_boxes and nrd_transfer (regrid.cu); a call holds the
-  // mutex while it uses it (several threads may transfer from one context)
+  // mutex while it uses it (several threads may transfer from one context: a
+  // call that finds it held allocates its own)
   std::mutex xfer_mu;
   void* d_xfer = nullptr;
   size_t xfer_bytes = 0;

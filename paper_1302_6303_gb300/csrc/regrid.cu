@@ -45,6 +45,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <optional>
 #include <string>
 #include <vector>
 
@@ -391,12 +392,38 @@ void xfer_done(nrd_ctx* c) {
   c->xfer_bytes = 0;
 }
 
+// One call's hold on that scratch; while another thread's call has it (several
+// may transfer from one context), an allocation of the call's own in its stream's
+// order, so that neither call waits for the other's work.
+struct Scratch {
+  nrd_ctx* c;
+  cudaStream_t s;
+  std::unique_lock<std::mutex> lock;
+  void* own = nullptr;
+  Scratch(nrd_ctx* ctx, cudaStream_t st) : c(ctx), s(st), lock(ctx->xfer_mu, std::try_to_lock) {}
+  Scratch(const Scratch&) = delete;
+  void* get(size_t bytes) {
+    if (lock.owns_lock()) return xfer_reserve(c, bytes);
+    if (cudaMallocAsync(&own, bytes, s) != cudaSuccess) {
+      cudaGetLastError();
+      own = nullptr;
+    }
+    return own;
+  }
+  ~Scratch() {
+    if (own) {
+      cudaFreeAsync(own, s);
+      cudaStreamSynchronize(s);   // the pool gives it back here
+    } else if (lock.owns_lock()) {
+      xfer_done(c);   // before the lock is released
+    }
+  }
+};
+
 // the device fields and tables of one level
 struct RgDevice {
-  nrd_ctx* c;
-  std::lock_guard<std::mutex> lock;
-  explicit RgDevice(nrd_ctx* ctx) : c(ctx), lock(ctx->xfer_mu) {}
-  ~RgDevice() { xfer_done(c); }   // before the lock is released
+  Scratch scratch;
+  explicit RgDevice(nrd_ctx* ctx) : scratch(ctx, nullptr) {}
   // tables of the tagged cells and (unless the level covers the domain) of the
   // nestable cells, on the host; false when the device had no memory for it
   bool tables(const Hier& H, const uint8_t* tags, int bits, int buffer, int l, const int n[3],
@@ -407,7 +434,7 @@ struct RgDevice {
     const int nt = full ? 1 : 2;
     const size_t pad = (nn + 255) / 256 * 256;
     const size_t bytes = 6 * pad + nt * tab * sizeof(int) + 6 * boxes.size() * sizeof(int);
-    uint8_t* buf = (uint8_t*)xfer_reserve(c, bytes);
+    uint8_t* buf = (uint8_t*)scratch.get(bytes);
     if (!buf) return false;
     uint8_t *raw = buf, *in = raw + pad, *h1 = in + pad, *o1 = h1 + pad, *h2 = o1 + pad,
             *o2 = h2 + pad;
@@ -688,11 +715,15 @@ int nrd_transfer(nrd_ctx* src, nrd_ctx* dst, const double* u_src, double* u_dst,
   const bool comp = A.L > 1;
   const size_t comp_bytes = comp ? 2 * No * nvec * sizeof(double) : 0;
   const size_t slot_bytes = comp ? (size_t)A.lev[A.L - 2].ncell * sizeof(int) : 0;
-  std::unique_lock<std::mutex> lock(src->xfer_mu, std::defer_lock);
-  if (comp) lock.lock();   // until the call returns: its kernels have ended then
-  if (comp && !xfer_reserve(src, comp_bytes + slot_bytes)) {
-    dst->err = "allocation failed";
-    return NRD_ENOMEM;
+  std::optional<Scratch> scratch;   // until the call returns: its kernels have ended then
+  char* buf = nullptr;
+  if (comp) {
+    scratch.emplace(src, s);
+    buf = (char*)scratch->get(comp_bytes + slot_bytes);
+    if (!buf) {
+      dst->err = "allocation failed";
+      return NRD_ENOMEM;
+    }
   }
   OldCells O{};
   O.L = A.L;
@@ -704,8 +735,8 @@ int nrd_transfer(nrd_ctx* src, nrd_ctx* dst, const double* u_src, double* u_dst,
   dst->timer.begin(NRD_TK_TRANSFER, s);
   if (comp) {
     const int lp = A.L - 2;
-    double* d_comp = (double*)src->d_xfer;
-    int* slot = (int*)((char*)src->d_xfer + comp_bytes);
+    double* d_comp = (double*)buf;
+    int* slot = (int*)(buf + comp_bytes);
     cudaMemcpyAsync(d_comp, u_src, comp_bytes, cudaMemcpyDeviceToDevice, s);
     launch_average_down(A, d_comp, 2 * nvec, (int)No, s);
     cudaMemsetAsync(slot, 0xff, slot_bytes, s);
@@ -721,7 +752,6 @@ int nrd_transfer(nrd_ctx* src, nrd_ctx* dst, const double* u_src, double* u_dst,
                                                  B.N, (int)No, nvec, old, u_dst);
   dst->timer.end(NRD_TK_TRANSFER, s);
   const cudaError_t e = cudaStreamSynchronize(s);
-  if (comp) xfer_done(src);
   if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) {
     dst->err = "transfer kernel failed";
     return NRD_ECUDA;

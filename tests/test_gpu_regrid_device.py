@@ -6,6 +6,7 @@ several vectors, repeated calls with growing scratch.  Boxes are integers and
 must be equal; the transfer's bound is that of the other transfer tests,
 1e-14 of max |u| (two FP64 operations per axis)."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -134,3 +135,39 @@ def test_tags_from_another_stream(nrd, cluster):
     if cluster == "tag default":
         got = boxes(tags)
     assert got == exp
+
+
+def test_transfer_does_not_wait_for_another(nrd):
+    """A transfer returns while another thread's, from the same context, still
+    waits for earlier work on its own stream."""
+    rng = np.random.default_rng(6)
+    n0 = (17, 12, 9)
+    a, b = random_hierarchy(rng, n0, 2), random_hierarchy(rng, n0, 3)
+    ca, cb = ctx_for(nrd, a), [ctx_for(nrd, b), ctx_for(nrd, b)]
+    u = dev(rng.uniform(0.1, 2.0, 2 * a.ncells))
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    exp = []
+    for s, c in zip(streams, cb):   # kernels loaded, output memory in each stream's pool
+        with torch.cuda.stream(s):
+            exp.append(ca.transfer_to(c, u).cpu())
+    torch.cuda.synchronize()
+    begun, ended, got = threading.Event(), threading.Event(), [None, None]
+
+    def late():
+        with torch.cuda.stream(streams[0]):
+            torch.cuda._sleep(4_000_000_000)   # about two seconds
+            begun.set()
+            got[0] = ca.transfer_to(cb[0], u)
+        ended.set()
+
+    th = threading.Thread(target=late)
+    th.start()
+    begun.wait()
+    time.sleep(0.3)
+    with torch.cuda.stream(streams[1]):
+        got[1] = ca.transfer_to(cb[1], u)
+    first = not ended.is_set()
+    th.join()
+    torch.cuda.synchronize()
+    assert first
+    assert all(torch.equal(g.cpu(), e) for g, e in zip(got, exp))
