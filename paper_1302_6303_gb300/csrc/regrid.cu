@@ -25,8 +25,8 @@
 // recursion accepts them (lower part first).
 //
 // The tagged and nestable fields of a level and their summed-area tables are
-// formed on the device (scatter, box filters, scans); the recursion reads the
-// tables on the host, 8 entries per count.
+// formed on the device (scatter, box filters, scans), for small levels on the
+// host; the recursion reads the tables on the host, 8 entries per count.
 //
 // nrd_transfer: conservative limited-linear transfer of state vectors from an
 // old to a new hierarchy, one device kernel that looks every new cell's source
@@ -254,6 +254,17 @@ struct Clusterer {
     out.push_back(b);
   }
 };
+
+// Small levels form their fields on the host: a copy of the tags and byte loops
+// (about 0.85 ns per cell and window cell) take less there than ten launches, the
+// tables' copy back (40 us) and 0.26 us per plane of running sums.  Whole calls for
+// 2 levels, host against device form (us): 4^3 23 against 57, 16^3 47 against 68
+// (buffer 8: 65 against 66), 18^3 59 against 70 (buffer 4: 74 against 69), 20^3 98
+// against 99, 24^3 101 against 82, 4x4x512 144 against 214.
+bool host_fields(const int n[3], int up, int buffer) {   // n of a level, `up` levels finer
+  const long cells = ((long)n[0] * n[1] * n[2]) << (3 * up), planes = ((long)n[1] + n[2]) << up;
+  return cells * (std::min(buffer, 8192) + 6L) <= 44000 + 300 * planes;
+}
 
 // ---- device side of the clustering: dense fields of one level
 struct Dims {
@@ -585,7 +596,7 @@ int nrd_regrid_boxes(nrd_ctx* c, const uint8_t* tags, int tag_bits, int buffer,
     return NRD_ECUDA;
   }
   const Hier& H = c->H;
-  std::vector<uint8_t> htags;   // filled when a level is done on the host
+  std::vector<uint8_t> htags;   // of the levels up to one done on the host
   const int n0[3] = {H.lev[0].n[0], H.lev[0].n[1], H.lev[0].n[2]};
   // tag of the current cell (l, q), or -1 if the current hierarchy has none
   auto cur_tag = [&](int l, const int q[3]) -> int {
@@ -603,11 +614,13 @@ int nrd_regrid_boxes(nrd_ctx* c, const uint8_t* tags, int tag_bits, int buffer,
       c->err = "nrd_regrid_boxes: a level is too large for int32 box counts";
       return NRD_EINVAL;
     }
-    // on the device; on the host where its memory does not allow the fields
+    // on the host where that is faster (host_fields) or the device's memory does
+    // not allow the fields
     std::vector<int> tables, osum_h;
     RgDevice dev{c};
     cudaError_t e = cudaSuccess;
-    const bool on_device = dev.tables(H, tags, tag_bits, buffer, l, n, levels[l], tables, e);
+    const bool on_device =
+        !host_fields(n, 0, buffer) && dev.tables(H, tags, tag_bits, buffer, l, n, levels[l], tables, e);
     if (on_device && (e != cudaSuccess || cudaGetLastError() != cudaSuccess)) {
       c->err = "clustering kernels failed";
       return NRD_ECUDA;
@@ -616,9 +629,14 @@ int nrd_regrid_boxes(nrd_ctx* c, const uint8_t* tags, int tag_bits, int buffer,
     const int* otab = nullptr;   // null: every cell is nestable
     if (on_device && l > 0) otab = tables.data() + (long)(n[0] + 1) * (n[1] + 1) * (n[2] + 1);
     if (!on_device) {
-      if (htags.empty()) {
-        htags.resize(H.N);
-        if (cudaMemcpy(htags.data(), tags, H.N, cudaMemcpyDeviceToHost) != cudaSuccess) {
+      // the tags of the levels up to this one, at once for all that will be done
+      // here (cells ascend by level)
+      int lt = std::min(l, H.L - 1);
+      while (lt + 1 < std::min(H.L, max_levels - 1) && host_fields(n, lt + 1 - l, buffer)) lt++;
+      const size_t need = (size_t)H.lev[lt].off + H.lev[lt].ncell;
+      if (htags.size() < need) {
+        htags.resize(need);
+        if (cudaMemcpy(htags.data(), tags, need, cudaMemcpyDeviceToHost) != cudaSuccess) {
           c->err = "copy of the tags failed";
           return NRD_ECUDA;
         }

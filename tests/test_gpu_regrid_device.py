@@ -171,3 +171,24 @@ def test_transfer_does_not_wait_for_another(nrd):
     torch.cuda.synchronize()
     assert first
     assert all(torch.equal(g.cpu(), e) for g, e in zip(got, exp))
+
+
+@pytest.mark.parametrize("n0,levels", [
+    ((16, 32, 16), 1), ((17, 32, 16), 1), ((33, 17, 15), 1), ((8193, 1, 1), 1), ((1, 97, 89), 1),
+    ((3, 4, 700), 1), ((40, 9, 25), 1), ((17, 18, 17), 1), ((9, 10, 700), 1), ((16, 32, 16), 2), ((17, 32, 16), 2), ((40, 9, 25), 2)])
+def test_boxes_both_forms(nrd, n0, levels):
+    """Index spaces on both sides of the line between the host and the device
+    form of the fields (about 20^3 cells, fewer with a wider buffer, more for a
+    long box), level 0 on one and level 1 on the other among them, against the
+    oracle."""
+    rng = np.random.default_rng(sum(n0) + levels)
+    h = W.uniform(n0) if levels == 1 else random_hierarchy(rng, n0, 2, count=2, side_lo=2,
+                                                           side_hi=4)
+    tags = (rng.random(h.ncells) < 0.01).astype(np.uint8) * 2
+    ctx = ctx_for(nrd, h)
+    for buf, eff, mn, mx, ml in [(0, 0.6, 2, 16, 2), (1, 0.7, 4, 32, 2 + (levels == 2)),
+                                 (5, 0.7, 4, 16, 2)]:
+        got = ctx.regrid_boxes(dev(tags), 2, buf, eff, mn, mx, ml)
+        exp = R.regrid_boxes(h, tags, tag_bits=2, buffer=buf, efficiency=eff, min_side=mn,
+                             max_side=mx, max_levels=ml)
+        assert as_lists(got) == as_lists(exp)
