@@ -868,7 +868,12 @@ struct JvArgs {
 // FP64 issue rate, the bound left, and 0.63 of HBM.  The row's order costs
 // 0.04 ms against own entries first, whose rounding error is a fifth larger
 // (2.5e-16 in the 2-norm against 2.1e-16 here, 2.2e-16 in flux form).
-__global__ void __launch_bounds__(256, 6) k_jv_frozen(JvArgs A) {
+// MINB < 6 (few tiles, launch_jv_frozen): the loads of several faces in flight,
+// and every cell by the boundary's path, since the cells of small patches mostly
+// take it and a warp holding both takes them in turn.
+template <int MINB>
+__global__ void __launch_bounds__(256, MINB) k_jv_frozen(JvArgs A) {
+  constexpr bool FEW = MINB < 6;
   const int N = A.N, G = A.G;
   double a0 = A.a0, dt = A.dt;
   if (A.par) {
@@ -902,7 +907,7 @@ __global__ void __launch_bounds__(256, 6) k_jv_frozen(JvArgs A) {
     double LE = soft_mul_any(J.cen[N + idx], vTc), LT = 0.0;
     const bool inner = i > 0 && i < nx - 1 && j > 0 && j < ny - 1 && k > 0 && k < nz - 1;
     const long NS = 3L * N + G;
-    if (inner && m == 0) {
+    if (!FEW && inner && m == 0) {
       const long st[3] = {1, nx, s2};
 #pragma unroll
       for (int d = 0; d < 3; d++) {
@@ -916,6 +921,51 @@ __global__ void __launch_bounds__(256, 6) k_jv_frozen(JvArgs A) {
         LE = fma(jh[NS], vE[hi], LE);
         LE = fma(jh[2 * NS], th, LE);
         LT = fma(jh[4 * NS], th, LT);
+      }
+    } else if (FEW) {
+      // Every face's kind first, then the loads without branches, so that those of
+      // several faces are in flight: one face after the other, each a chain of
+      // dependent loads, took most of the time of a few small patches.
+      const int pos[3] = {i, j, k};
+      auto ghost = [&](int f) {
+        const int d = f >> 1;
+        return P.goff + P.fo[f] + pos[(d + 1) % 3] + P.n[(d + 1) % 3] * pos[(d + 2) % 3];
+      };
+      unsigned bnd = 0, use = 0, cf = 0;   // bit f: patch boundary; enters the row; coarse-fine
+#pragma unroll
+      for (int f = 0; f < 6; f++) {
+        if (pos[f >> 1] == (f & 1 ? P.n[f >> 1] - 1 : 0)) bnd |= 1u << f;
+        const uint8_t gt = (bnd >> f & 1) ? A.gtype[ghost(f)] : GT_SIBLING;
+        // (not: faces taken by flux matching; physical ones, own entries only)
+        if (!(m & (2 << f)) && gt != GT_NEUMANN && gt != GT_ROBIN) use |= 1u << f;
+        if (gt == GT_CF) cf |= 1u << f;
+      }
+#pragma unroll
+      for (int f = 0; f < 6; f++) {
+        const int d = f >> 1, hi = f & 1;
+        const long st = (d == 0) ? 1L : (d == 1 ? (long)nx : s2);
+        const bool b = bnd >> f & 1, on = use >> f & 1;
+        const long n = hi ? idx + st : idx - st;
+        const double* jf = J.jc + (b ? 3L * N + ghost(f) : (long)d * N + (hi ? n : idx));
+        const double* nv = b ? A.gv + ghost(f) : vE + n;
+        const double cE = on ? jf[hi ? NS : 0] : 0.0, cX = on ? jf[2 * NS] : 0.0;
+        const double cT = on ? jf[hi ? 4 * NS : 3 * NS] : 0.0;
+        const double nE = on ? nv[0] : 0.0, nT = on ? nv[b ? G : N] : 0.0;
+        LE = fma(hi ? cE : -cE, nE, LE);
+        LE = fma(hi ? cX : -cX, nT, LE);
+        LT = fma(hi ? cT : -cT, nT, LT);
+      }
+      cf &= use;
+#pragma unroll
+      for (int f = 0; f < 6; f++) {
+        if (!(cf >> f & 1)) continue;
+        const int hi = f & 1, g = ghost(f);
+        const double* jf = J.jc + 3L * N + g;
+        const double nE = A.gv[g], nT = A.gv[G + g];
+        const double Ea = hi ? vEc : nE, Eb = hi ? nE : vEc;
+        const double Ta = hi ? vTc : nT, Tb = hi ? nT : vTc;
+        A.cf[g] = fma(jf[0], Ea, fma(jf[NS], Eb, jf[2 * NS] * (Ta + Tb)));
+        A.cf[G + g] = fma(jf[3 * NS], Ta, jf[4 * NS] * Tb);
       }
     } else {
       const int pos[3] = {i, j, k};
@@ -1331,7 +1381,16 @@ void launch_jv_frozen(const Hier& H, const StencilIO& io, cudaStream_t s) {
   a.par = io.par;
   const int nt = (int)H.tiles.size();
   const int cells = H.tile_x * H.tile_y * H.tile_z;
-  k_jv_frozen<<<nt, std::min(256, cells), 0, s>>>(a);
+  const int bs = std::min(256, cells);
+  // Few tiles are bound by the latency of a cell's chain of loads, not by issue:
+  // registers for more of them instead of blocks.  Durations with cold caches, us,
+  // six blocks per SM -> this: 8^3 with fine patches (18 tiles) 17.1 -> 12.4, base
+  // 16^3 + fine band (160 tiles) 13.6 -> 9.5; base 32^3 + band in 8x8x4 tiles 14.6
+  // -> 11.3, 64^3 in 8x8x8 tiles (968) 26.2 -> 19.4.  Beyond, 64^3 in 8x8x4 tiles
+  // (1480): 23.7 against 24.9 with four.
+  if (nt <= 2 * 152) k_jv_frozen<2><<<nt, bs, 0, s>>>(a);
+  else if (nt <= 8 * 152) k_jv_frozen<4><<<nt, bs, 0, s>>>(a);
+  else k_jv_frozen<6><<<nt, bs, 0, s>>>(a);
 }
 
 void launch_tag(const Hier& H, const double* E, const double* gE, double thr_c, double thr_g,
