@@ -421,8 +421,8 @@ constexpr int min_blocks(int mode) {
 // idles on a cell outside its patch.  Without CMP the extents are the
 // compile-time shape (fewer registers: the form for hierarchies without
 // such tiles).
-template <int MODE, int TX, int TY, int TZ, bool CMP = false>
-__global__ void __launch_bounds__(256, min_blocks(MODE)) k_stencil(StArgs A) {
+template <int MODE, int TX, int TY, int TZ, bool CMP, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_stencil(StArgs A) {
   constexpr int HX = TX + 2, HY = TY + 2, HZ = TZ + 2;
   constexpr int NH = HX * HY * HZ;
   constexpr int NFX = (TX + 1) * TY * TZ, NFY = TX * (TY + 1) * TZ, NFZ = TX * TY * (TZ + 1);
@@ -1240,33 +1240,33 @@ size_t stencil_smem() {
   return d * sizeof(double);
 }
 
-template <int MODE, int TX, int TY, int TZ, bool CMP>
+template <int MODE, int TX, int TY, int TZ, bool CMP, int MINB>
 void run_stencil(const StArgs& a, cudaStream_t s) {
   size_t sm = stencil_smem<MODE, TX, TY, TZ>();
   static bool init = false;
   if (!init) {
-    cudaFuncSetAttribute(k_stencil<MODE, TX, TY, TZ, CMP>,
+    cudaFuncSetAttribute(k_stencil<MODE, TX, TY, TZ, CMP, MINB>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     init = true;
   }
   // one tile per CTA: the block scheduler balances tiles of uneven cost
   int grid = a.ntiles;
   if (grid < 1) return;
-  k_stencil<MODE, TX, TY, TZ, CMP><<<grid, 256, sm, s>>>(a);
+  k_stencil<MODE, TX, TY, TZ, CMP, MINB><<<grid, 256, sm, s>>>(a);
 }
 
-template <int MODE, bool CMP = false>
+template <int MODE, bool CMP = false, int MINB = min_blocks(MODE)>
 void dispatch_tile(const StArgs& a, int tx, int ty, int tz, cudaStream_t s) {
-  if (tx == 32 && ty == 8 && tz == 4) run_stencil<MODE, 32, 8, 4, CMP>(a, s);
-  else if (tx == 32 && ty == 4 && tz == 8) run_stencil<MODE, 32, 4, 8, CMP>(a, s);
-  else if (tx == 32 && ty == 2 && tz == 4) run_stencil<MODE, 32, 2, 4, CMP>(a, s);
-  else if (tx == 16 && ty == 8 && tz == 4) run_stencil<MODE, 16, 8, 4, CMP>(a, s);
-  else if (tx == 16 && ty == 4 && tz == 8) run_stencil<MODE, 16, 4, 8, CMP>(a, s);
-  else if (tx == 16 && ty == 8 && tz == 8) run_stencil<MODE, 16, 8, 8, CMP>(a, s);
-  else if (tx == 16 && ty == 4 && tz == 4) run_stencil<MODE, 16, 4, 4, CMP>(a, s);
-  else if (tx == 8 && ty == 8 && tz == 8) run_stencil<MODE, 8, 8, 8, CMP>(a, s);
-  else if (tx == 8 && ty == 8 && tz == 4) run_stencil<MODE, 8, 8, 4, CMP>(a, s);
-  else run_stencil<MODE, 32, 4, 4, CMP>(a, s);
+  if (tx == 32 && ty == 8 && tz == 4) run_stencil<MODE, 32, 8, 4, CMP, MINB>(a, s);
+  else if (tx == 32 && ty == 4 && tz == 8) run_stencil<MODE, 32, 4, 8, CMP, MINB>(a, s);
+  else if (tx == 32 && ty == 2 && tz == 4) run_stencil<MODE, 32, 2, 4, CMP, MINB>(a, s);
+  else if (tx == 16 && ty == 8 && tz == 4) run_stencil<MODE, 16, 8, 4, CMP, MINB>(a, s);
+  else if (tx == 16 && ty == 4 && tz == 8) run_stencil<MODE, 16, 4, 8, CMP, MINB>(a, s);
+  else if (tx == 16 && ty == 8 && tz == 8) run_stencil<MODE, 16, 8, 8, CMP, MINB>(a, s);
+  else if (tx == 16 && ty == 4 && tz == 4) run_stencil<MODE, 16, 4, 4, CMP, MINB>(a, s);
+  else if (tx == 8 && ty == 8 && tz == 8) run_stencil<MODE, 8, 8, 8, CMP, MINB>(a, s);
+  else if (tx == 8 && ty == 8 && tz == 4) run_stencil<MODE, 8, 8, 4, CMP, MINB>(a, s);
+  else run_stencil<MODE, 32, 4, 4, CMP, MINB>(a, s);
 }
 
 // the compact-cell form where the hierarchy has ragged tiles, for the launches
@@ -1332,7 +1332,14 @@ void launch_stencil(const Hier& H, const ModelParams& mp, int mode, const Stenci
   a.soft = soft_constants(H, a.lh);
   a.io = io;
   if (mode == ST_RESIDUAL) {
-    dispatch_tile<ST_RESF>(a, H.tile_x, H.tile_y, H.tile_z, s);
+    // eight blocks per SM cap the registers: at up to that many tiles in all the
+    // face launch is faster with four (us: 16^3 in 32x4x4 tiles 12.2 -> 10.1, 64^3 in
+    // 8x8x8 43.3 -> 38.6; 96^3, 2,184 tiles, 92.8 against 94.1 with four, 256^3 1368
+    // against 1484)
+    if (a.ntiles <= 8 * 152)
+      dispatch_tile<ST_RESF, false, 4>(a, H.tile_x, H.tile_y, H.tile_z, s);
+    else
+      dispatch_tile<ST_RESF>(a, H.tile_x, H.tile_y, H.tile_z, s);
     dispatch_tile_h<ST_RESC>(H, a, s);
   } else if (mode == ST_JV) {
     dispatch_tile<ST_JV>(a, H.tile_x, H.tile_y, H.tile_z, s);

@@ -1,7 +1,7 @@
 """The frozen Jv has forms for hierarchies of few tiles (up to 304 and 1,216 of
-them); each against the oracle on either side of the lines, on whole and ragged
-boxes and on patches, with and without Robin faces.  Tolerance 1e-12 of each cell's term
-scale, as in the parity tests."""
+them), the residual one (up to 1,216); each against the oracle on either side of
+the lines, on whole and ragged boxes and on patches, with and without Robin
+faces.  Tolerance 1e-12 of each cell's term scale, as in the parity tests."""
 import numpy as np
 import pytest
 
@@ -56,3 +56,22 @@ def test_frozen_jv(nrd, name):
     o = Oracle(h, z)
     S = o.jv_scale(u, v, a0, dt)
     assert np.all(np.abs(J - o.jv_analytic(u, v, a0, dt)) <= 1e-12 * S + 1e-300)
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_residual(nrd, name):
+    mk, tile = CASES[name]
+    h = mk()
+    z = W.material_from_cubes(h, [((2, 2, 2), 3, 10.0)])
+    u = W.front_state(h, seed=2, noise=0.1)
+    b = u * (1 + 0.05 * np.random.default_rng(4).uniform(-1, 1, u.size))
+    ctx = nrd.Context(nmg=1, tile_x=tile[0], tile_y=tile[1], tile_z=tile[2])
+    ctx.set_hierarchy_from(h)
+    ctx.set_material(dev(z))
+    a0, dt = 1.5, 3e-3
+    F = ctx.residual(dev(u), dev(b), a0, dt)
+    o = Oracle(h, z)
+    S = o.residual_scale(u, b, a0, dt)
+    assert np.all(np.abs(F.cpu().numpy() - o.residual(u, b, a0, dt)) <= 1e-12 * S + 1e-300)
+    # the linearisation's residual has the same bits
+    assert torch.equal(ctx.linearise(dev(u), dev(b), a0, dt), F)
