@@ -632,10 +632,27 @@ struct VLev {
   int N, G;
 };
 
-// body(item) for the tiles blockIdx.x, blockIdx.x + gridDim.x, ... of a list
-template <class F>
+// body(item) for the tiles blockIdx.x, blockIdx.x + gridDim.x, ... of a list.
+// WHOLE: an item is loaded at once, 16 bytes at a time, instead of by the fields
+// the body reads.  Composite residual in FP64 on 250 patches (5.7M cells) 401 ->
+// 393 us, damped Jacobi sweep 441 -> 437 in FP64, 113 -> 104 in FP32; the FP32
+// composite residual takes 115 us so and 113 by fields, the red-black sweep the
+// same either way.
+template <bool WHOLE, class F>
 __device__ __forceinline__ void tile_loop(int ntl, const VItem* __restrict__ items, F body) {
-  for (int tt = blockIdx.x; tt < ntl; tt += gridDim.x) body(items[tt]);
+  for (int tt = blockIdx.x; tt < ntl; tt += gridDim.x) {
+    if (WHOLE) {
+      constexpr int W = sizeof(VItem) / sizeof(int4);
+      static_assert(sizeof(VItem) % sizeof(int4) == 0, "");
+      union { int4 q[W]; VItem it; } u;
+      const int4* src = reinterpret_cast<const int4*>(items + tt);
+#pragma unroll
+      for (int k = 0; k < W; k++) u.q[k] = __ldg(src + k);
+      body(u.it);
+    } else {
+      body(items[tt]);
+    }
+  }
 }
 
 // ghost slot of face fc of cell (a, b) in the face's (t1, t2) coordinates
@@ -731,7 +748,7 @@ __global__ void __launch_bounds__(VTHREADS) k_lsmooth(int ntl, VLev<P> V, int t0
                                                       P* __restrict__ e,
                                                       const P* __restrict__ f,
                                                       P* __restrict__ u) {
-  tile_loop(ntl, V.vt + t0, [&](const VItem& it) {
+  tile_loop<(sizeof(P) > 4)>(ntl, V.vt + t0, [&](const VItem& it) {
     k_lsmooth_tile<P, ZERO, ADD>(it, V, colour, e, f, u);
   });
 }
@@ -817,7 +834,7 @@ __global__ void __launch_bounds__(FTHREADS) k_ljacobi(int ntl, VLev<P> V, int t0
                                                       P* __restrict__ ed,
                                                       const P* __restrict__ f,
                                                       P* __restrict__ u) {
-  tile_loop(ntl, V.vt + t0, [&](const VItem& it) {
+  tile_loop<true>(ntl, V.vt + t0, [&](const VItem& it) {
     k_ljacobi_tile<P, ZERO, ADD>(it, V, omega, es, ed, f, u);
   });
 }
@@ -907,7 +924,8 @@ template <class P>
 __global__ void __launch_bounds__(FTHREADS) k_cresid(int ntl, VLev<P> V, const P* __restrict__ u,
                                                      const P* __restrict__ f,
                                                      P* __restrict__ r, P* __restrict__ cf) {
-  tile_loop(ntl, V.vt, [&](const VItem& it) { k_cresid_tile<P>(it, V, u, f, r, cf); });
+  tile_loop<(sizeof(P) > 4)>(ntl, V.vt,
+                             [&](const VItem& it) { k_cresid_tile<P>(it, V, u, f, r, cf); });
 }
 
 // flux matching of the composite operator (each coarse cell with coarse-fine
@@ -1017,7 +1035,7 @@ __global__ void __launch_bounds__(FTHREADS) k_vprolong(int ntl, VLev<P> V, int t
                                                        int cn0, int cn1, int cn2,
                                                        const P* __restrict__ src,
                                                        P* __restrict__ pv, P* __restrict__ u) {
-  tile_loop(ntl, V.vt + t0, [&](const VItem& it) {
+  tile_loop<(sizeof(P) > 4)>(ntl, V.vt + t0, [&](const VItem& it) {
     k_vprolong_tile<P, PV>(it, V, cmap, cn0, cn1, cn2, src, pv, u);
   });
 }
