@@ -104,3 +104,48 @@ def test_window(nrd, name, tile, outside):
     J = ctx.jv(dev(u), dev(v), a0, dt, mode=nrd.JV_FROZEN).cpu().numpy()
     Sj = o.jv_scale(u, v, a0, dt)
     assert np.all(np.abs(J - o.jv_analytic(u, v, a0, dt)) <= 1e-12 * Sj + 1e-300)
+
+
+VJP_HIERS = {
+    "box8": lambda: W.uniform(8),
+    "ragged": lambda: W.uniform((20, 12, 7)),
+    "amr3": lambda: W.tiny_amr(8, True),
+    "boundary": lambda: W.boundary_amr(8),     # patches on Robin and coarse-fine faces at once
+}
+
+
+@pytest.mark.parametrize("outside", ["none", "some", "all"])
+@pytest.mark.parametrize("tile", [(8, 8, 8), (32, 4, 4)])
+@pytest.mark.parametrize("name", list(VJP_HIERS))
+def test_window_transpose(nrd, name, tile, outside):
+    """The transposed product and the material partials with no, some and all
+    cells outside the window, and both products on vectors whose entries leave
+    the range of their integer products (2^-480 .. 2^480) and are zero."""
+    h = VJP_HIERS[name]()
+    z = W.material_from_cubes(h, [((2, 2, 2), 3, 10.0)])
+    u = W.front_state(h, seed=2, noise=0.1)
+    N = h.ncells
+    rng = np.random.default_rng(4)
+    if outside == "some":
+        u[rng.integers(0, N, max(1, N // 40))] = 1e-22
+    elif outside == "all":
+        u[:N] *= 1e-21
+    ctx = nrd.Context(nmg=1, tile_x=tile[0], tile_y=tile[1], tile_z=tile[2])
+    ctx.set_hierarchy_from(h)
+    ctx.set_material(dev(z))
+    o = Oracle(h, z)
+    a0, dt = 1.5, 3e-3
+    ctx.linearise(dev(u), dev(u * 0.95), a0, dt)
+    w = W.random_direction(h, 7)
+    JTw, dz = ctx.vjp(dev(w), a0, dt)
+    JTo, dzo, S = o.vjp(u, w, a0, dt)
+    assert np.all(np.abs(JTw.cpu().numpy() - JTo) <= 1e-12 * S + 1e-300)
+    assert np.abs(dz.cpu().numpy() - dzo).max() <= 1e-11 * np.abs(dzo).max()
+    wide = w * 10.0 ** rng.choice([-200.0, -150.0, 0.0, 0.0, 160.0], w.size)
+    wide[rng.integers(0, w.size, w.size // 10)] = 0.0
+    JTw, _ = ctx.vjp(dev(wide), a0, dt, want_dz=False)
+    JTo, _, S = o.vjp(u, wide, a0, dt, with_dz=False)
+    assert np.all(np.abs(JTw.cpu().numpy() - JTo) <= 1e-12 * S + 1e-300)
+    J = ctx.jv(dev(u), dev(wide), a0, dt, mode=nrd.JV_FROZEN).cpu().numpy()
+    S = o.jv_scale(u, wide, a0, dt)
+    assert np.all(np.abs(J - o.jv_analytic(u, wide, a0, dt)) <= 1e-12 * S + 1e-300)
