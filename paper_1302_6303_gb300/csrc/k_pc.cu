@@ -556,7 +556,7 @@ __device__ __forceinline__ P tri_interp(const P* src, int cn0, int cn1, int cn2,
 // result is bit-identical to tri_interp per fine cell.  grid (coarse x / 8,
 // y / 8, 2 fields x z / 4), 256 threads.
 constexpr int PX = 8, PY = 8, PZ = 4;
-template <class P, bool PAIR>
+template <class P>
 __global__ void __launch_bounds__(PX * PY * PZ) k_bprolong(const P* ec, int cn0, int cn1,
                                                             int cn2, BoxK<P> F, P* out) {
   const int ntz = gridDim.z >> 1;
@@ -578,8 +578,10 @@ __global__ void __launch_bounds__(PX * PY * PZ) k_bprolong(const P* ec, int cn0,
     for (int y = 0; y < 3; y++)
 #pragma unroll
       for (int x = 0; x < 3; x++) c[z][y][x] = src[cx[x] + cn0 * (cy[y] + cn1 * cz[z])];
-  // the two children of a row are read and written as one pair (they start at
-  // an even cell; PAIR: the arrays are aligned to pairs)
+  // the two children of a row are read and written as one pair: they start at an
+  // even cell, and a level with a coarser one has even sides (pc_alloc), so that
+  // rows and fields start there too.  Over the launches of a V-cycle at 256^3 125
+  // -> 104 us against one cell at a time.
   struct alignas(2 * sizeof(P)) Pair { P a, b; };
 #pragma unroll
   for (int sz = 0; sz < 2; sz++)
@@ -601,13 +603,8 @@ __global__ void __launch_bounds__(PX * PY * PZ) k_bprolong(const P* ec, int cn0,
         }
       }
       const long idx = fo + i + F.n0 * (j + (long)F.n1 * k);
-      if (PAIR) {
-        const Pair e = *reinterpret_cast<const Pair*>(F.e + idx);
-        *reinterpret_cast<Pair*>(out + idx) = {e.a + v[0], e.b + v[1]};
-      } else {
-        out[idx] = F.e[idx] + v[0];
-        if (i + 1 < F.n0) out[idx + 1] = F.e[idx + 1] + v[1];
-      }
+      const Pair e = *reinterpret_cast<const Pair*>(F.e + idx);
+      *reinterpret_cast<Pair*>(out + idx) = {e.a + v[0], e.b + v[1]};
     }
 }
 
@@ -2116,14 +2113,8 @@ void gmg_vcycle(PcState* ps, const Hier& H, int m, cudaStream_t s) {
       (jac || fused_sweeps<P>(ps, m)) && ps->nu2 > 0 && start_in_scratch(ps->nu2);
   const dim3 gp((C.n[0] + PX - 1) / PX, (C.n[1] + PY - 1) / PY, 2 * ((C.n[2] + PZ - 1) / PZ));
   P* to = to_scratch ? scratch : V.e;
-  // pairs of cells: rows and fields of even length (the arrays themselves are
-  // allocations, aligned far beyond a pair).  V-cycle at 256^3: 125 -> 104 us in all.
-  if (V.n0 % 2 == 0 && V.vfs % 2 == 0)
-    k_bprolong<P, true><<<gp, PX * PY * PZ, 0, s>>>((const P*)ps->be[m + 1], C.n[0], C.n[1],
-                                                    C.n[2], V, to);
-  else
-    k_bprolong<P, false><<<gp, PX * PY * PZ, 0, s>>>((const P*)ps->be[m + 1], C.n[0], C.n[1],
-                                                     C.n[2], V, to);
+  k_bprolong<P><<<gp, PX * PY * PZ, 0, s>>>((const P*)ps->be[m + 1], C.n[0], C.n[1], C.n[2], V,
+                                            to);
   if (ps->nu2 == 0) {
     if (m == 0 && H.L > 1) add_level<P>(ps, H, 0, s);
   } else if (jac) {

@@ -414,13 +414,12 @@ constexpr int min_blocks(int mode) {
   }
 }
 
-// CMP: the cell loops (and the fused forms' face loop) run over the cells of
-// a tile inside its patch only, with index arithmetic in the tile's runtime
-// extent; used where the hierarchy has tiles narrower than the tile shape
-// (patches whose sides are not multiples of it), so that no lane of a warp
-// idles on a cell outside its patch.  Without CMP the extents are the
-// compile-time shape (fewer registers: the form for hierarchies without
-// such tiles).
+// CMP: the cell launches' loop runs over the cells of a tile inside its patch
+// only, with index arithmetic in the tile's runtime extent; used where the
+// hierarchy has tiles narrower than the tile shape (patches whose sides are not
+// multiples of it), so that no lane of a warp idles on a cell outside its patch.
+// Without CMP the extents are the compile-time shape (fewer registers: the form
+// for hierarchies without such tiles).
 template <int MODE, int TX, int TY, int TZ, bool CMP, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_stencil(StArgs A) {
   constexpr int HX = TX + 2, HY = TY + 2, HZ = TZ + 2;
@@ -623,9 +622,7 @@ __global__ void __launch_bounds__(256, MINB) k_stencil(StArgs A) {
     const int nbx = (FACES && tile.i0 + ex == nx) ? ey * tzl : 0;
     const int nby = (FACES && tile.j0 + ey == ny) ? ex * tzl : 0;
     const int nbz = (FACES && tile.k1 == nz) ? ex * ey : 0;
-    const int nfxe = (ex + 1) * ey * tzl, nfye = ex * (ey + 1) * tzl;
-    const int nfaces = FACES ? 3 * nlow + nbx + nby + nbz
-                             : (CMP ? nfxe + nfye + ex * ey * (tzl + 1) : NFX + NFY + NFZ);
+    const int nfaces = FACES ? 3 * nlow + nbx + nby + nbz : NFX + NFY + NFZ;
     auto faces = [&](auto softc) {
     constexpr bool SOFT = decltype(softc)::value;
     for (int f = threadIdx.x; f < nfaces; f += blockDim.x) {
@@ -649,24 +646,6 @@ __global__ void __launch_bounds__(256, MINB) k_stencil(StArgs A) {
         } else {
           q -= nby;
           dir = 2; fk = tzl; fi = q % ex; fj = q / ex;
-        }
-      } else if (CMP) {
-        // the faces of the tile's cells inside the patch, each written to its
-        // full-tile slot (the cell loop reads them there)
-        int q = f;
-        if (q < nfxe) {
-          dir = 0; fi = q % (ex + 1); fj = (q / (ex + 1)) % ey; fk = q / ((ex + 1) * ey);
-          slot = fi + (TX + 1) * (fj + TY * fk);
-          outE = fxE; outT = fxT;
-        } else if ((q -= nfxe) < nfye) {
-          dir = 1; fi = q % ex; fj = (q / ex) % (ey + 1); fk = q / (ex * (ey + 1));
-          slot = fi + TX * (fj + (TY + 1) * fk);
-          outE = fyE; outT = fyT;
-        } else {
-          q -= nfye;
-          dir = 2; fi = q % ex; fj = (q / ex) % ey; fk = q / (ex * ey);
-          slot = fi + TX * (fj + TY * fk);
-          outE = fzE; outT = fzT;
         }
       } else if (f < NFX) {
         dir = 0; slot = f;
@@ -796,10 +775,8 @@ __global__ void __launch_bounds__(256, MINB) k_stencil(StArgs A) {
     __syncthreads();
     if (FACES) continue;   // the cell launch forms the balance
     // ---- cell balance
-    const int fex = CMP ? ex : TX, fey = CMP ? ey : TY;
-    const int nce = CMP ? ex * ey * tzl : NC;
-    for (int c = threadIdx.x; c < nce; c += blockDim.x) {
-      int ci = c % fex, cj = (c / fex) % fey, ck = c / (fex * fey);
+    for (int c = threadIdx.x; c < NC; c += blockDim.x) {
+      int ci = c % TX, cj = (c / TX) % TY, ck = c / (TX * TY);
       int i = tile.i0 + ci, j = tile.j0 + cj, k = tile.k0 + ck;
       if (i >= nx || j >= ny || k >= tile.k1) continue;
       int idx = P.off + i + nx * (j + ny * k);
@@ -1269,8 +1246,7 @@ void dispatch_tile(const StArgs& a, int tx, int ty, int tz, cudaStream_t s) {
   else run_stencil<MODE, 32, 4, 4, CMP, MINB>(a, s);
 }
 
-// the compact-cell form where the hierarchy has ragged tiles, for the launches
-// of the Newton and Krylov loops (the cell launches and the frozen Jv)
+// the cell launches: the compact-cell form where the hierarchy has ragged tiles
 template <int MODE>
 void dispatch_tile_h(const Hier& H, const StArgs& a, cudaStream_t s) {
   if (H.ragged) dispatch_tile<MODE, true>(a, H.tile_x, H.tile_y, H.tile_z, s);
