@@ -119,17 +119,17 @@ JV_BYTES_PER_CELL = 185.0
 # (single256: captured on the same layout at 128^3, 2,097,152 cells, and
 # scaled by the cells, x8: these stencils stream their inputs once; the
 # linearisation's face and cell launches 58.0 + 400.0 + 441.9 + 129.1 MB,
-# the frozen Jv 356.0 + 46.9 MB)
+# the frozen Jv 355.9 + 49.1 MB)
 TRAFFIC = {
     "amr2_base64": {"linearise": None, "jv": None},
     "batching_base128": {"linearise": None, "jv": None},
     "single256": {"linearise": 8 * (58.0 + 400.0 + 441.9 + 129.1) * 1e6,
-                  "jv": 8 * (356.0 + 46.9) * 1e6},
+                  "jv": 8 * (355.9 + 49.1) * 1e6},
 }
 # FP64-pipe instructions per cell measured by ncu (sm__inst_executed_pipe_fp64,
-# same capture): linearisation 67.1 + 40.0, frozen Jv 24.6 (about half the
+# same capture): linearisation 67.1 + 40.0, frozen Jv 25.6 (about half the
 # products run on the integer pipe and are not in these counts)
-LIN_INST_NCU, JV_INST_NCU = 67.1 + 40.0, 24.6
+LIN_INST_NCU, JV_INST_NCU = 67.1 + 40.0, 25.6
 # Algorithmic DRAM bytes per leaf cell of the linearisation as laid out here:
 # face launch reads E, T, z^3 (24 B) and writes per face slot (3 per cell) the
 # 5 FP64 Jacobian partials, the 2 scaled FP32 P1 coefficients and the 2 FP64
@@ -622,7 +622,7 @@ def regrid_leg(nrd, ctx, torch, h, z, r):
     k_ms, _ = cn.timing_read()["transfer"]
     cn.timing_enable(False)
     No, Nn, nvec = ctx.N, cn.N, 2
-    alg = 2 * 16 * nvec * No + 4 * Nn + 2 * 16 * nvec * Nn
+    alg = 2 * 16 * nvec * (No + Nn)
     # warm restart: the last step solved again (backward-Euler form from the
     # transferred u_{n-1}) from the transferred u_n
     un = moved[0].contiguous()
@@ -634,9 +634,9 @@ def regrid_leg(nrd, ctx, torch, h, z, r):
             "leaf_cells_new": cn.nleaf, "transfer_ms_total": transfer_ms,
             "transfer_kernel_ms": k_ms, "transfer_vectors": nvec,
             "transfer_gbs": alg / (k_ms * 1e-3) / 1e9 if k_ms > 0 else None,
-            "transfer_bytes": "copy of the old vectors (read+write) + 4 B source code per new "
-                              "cell + one read and one write per new value (the 44 B entries "
-                              "of reconstructed cells not counted)",
+            "transfer_bytes": "copy of the old vectors (read+write) + one read and one write "
+                              "per new value (the source look-ups and the further values of "
+                              "reconstructed cells not counted)",
             "resolve_ms": e0.elapsed_time(e1), "resolve_newton": st["newton_its"],
             "resolve_krylov": st["krylov_its"], "fnorm_after_transfer": st["fnorm0"],
             "fnorm_resolved": st["fnorm"]}
@@ -954,7 +954,7 @@ def main():
                             "ratio_to_analytic": tpc / RES_BYTES_PER_CELL,
                             "why": "reads the 5 stored FP64 partials per face and 4 own "
                                    "entries per cell instead of re-deriving them from E, T "
-                                   "and z (25 FP64 instructions per cell instead of about "
+                                   "and z (26 FP64 instructions per cell instead of about "
                                    "130)"}
     pc_ms, pc_n = kt["pc_apply"]
     t_pc = pc_ms / max(pc_n, 1) * 1e-3

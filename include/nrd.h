@@ -332,8 +332,8 @@ int nrd_tag(nrd_ctx* ctx, const double* u, double thr_c, double thr_g, double th
  *   it exceeds max_boxes, which returns NRD_EINVAL, as does a level whose
  *   index space has 2^31 cells or more).  The fields of a level (about 14 bytes
  *   per cell of its index space) are formed in device memory, on the host for
- *   small levels and when that is not to be had.  Works on the legacy default stream and
- *   synchronises. */
+ *   small levels and when that is not to be had.  Works on the legacy default
+ *   stream and synchronises. */
 int nrd_regrid_boxes(nrd_ctx* ctx, const uint8_t* tags, int tag_bits, int buffer,
                      double efficiency, int min_side, int max_side, int max_levels,
                      int max_boxes, int* nlevels_out, int* nboxes_out, int* boxes_out,

@@ -694,12 +694,13 @@ constexpr double kReorthFrac = 1e-4;
 // Every block sums the partials in the same order, so all take the same
 // branch.  Bound by latency on small vectors (loads, the reduction trees and
 // the grid barrier) and by the FP64 pipe and HBM together on large ones.  Per
-// call of a step's solves, against block trees per quantity and columns loaded
-// one after the other: 32^3 21.6 -> 12.9 us, base 64^3 + fine band (0.5M cells)
-// 52.3 -> 42.1 us, 256^3 647 -> 570 us.  always2: the second pass every time (CGS2; solves that need an
-// orthogonal basis to working precision, such as the adjoint's).  end (end.c
-// non-null): block 0 ends the Arnoldi step of the Newton graph while the others
-// form V[nv] (a one-thread kernel of 6 us and a launch less per iteration).
+// call of a step's solves (CUDA events), against block trees per quantity and
+// columns loaded one after the other: 32^3 21.7 -> 13.7 us, base 64^3 + fine band
+// (0.5M cells) 53.3 -> 42.5 us, 256^3 651 -> 551 us.  always2: the second pass
+// every time (CGS2; solves that need an orthogonal basis to working precision,
+// such as the adjoint's).  end (end.c non-null): block 0 ends the Arnoldi step of
+// the Newton graph while the others form V[nv] (a one-thread kernel of 6 us and a
+// launch less per iteration).
 __global__ void __launch_bounds__(RB, 3) k_orth_coop(LevW lw, double* __restrict__ w,
                                                    double* __restrict__ V, long stride, int N,
                                                    const int* jd, int add, double* pa, double* pb,

@@ -203,7 +203,7 @@ __device__ __forceinline__ float narrow_rn(double x) {
 // where SOFT (the same bits, see softfp.h).  Both pipes then take about the
 // same time.  Measured at 256^3 (8x8x8 tiles), against the plain formulas on the
 // FP64 pipe alone (45 and 26 instructions a face): the linearisation's face
-// launch 4.25 -> 2.16 ms, the residual's 2.66 -> 1.37 ms.
+// launch 4.25 -> 2.04 ms, the residual's 2.66 -> 1.37 ms.
 struct FaceCore {
   double Ts, dE, S, r, Q, X, lt, PE, y, dT, T25, PT;
 };
@@ -268,8 +268,9 @@ __device__ __forceinline__ FaceLin flux_lin(double Ea, double Eb, double Ta, dou
 // shared by the residual and the linearisation (bit-identical F); returns
 // 1/T and sigma for the partial derivatives.
 // (SOFT: E, T and z^3 in the soft window; the same bits either way.  At 256^3
-// the linearisation's cell launch 1.08 -> 0.72 ms, the residual's 0.89 ->
-// 0.63 ms.)
+// it took the residual's cell launch from 0.89 to 0.63 ms and the linearisation's
+// from 1.08 to 0.72; the latter takes 1.25 ms since it also sums the cell's own
+// Jacobian entries.)
 template <bool SOFT>
 __device__ __forceinline__ void cell_balance(double a0, double dt, double E, double T, double z3,
                                              double bE, double bT, double divE, double divT,
@@ -835,16 +836,18 @@ struct JvArgs {
   const double* par;
 };
 
-// Frozen Jv: out = a0 v - dt L v, one row sum per cell and field (24.6 FP64
+// Frozen Jv: out = a0 v - dt L v, one row sum per cell and field (25.6 FP64
 // instructions, counted) over the 19 coefficients of the cell; fine-side coarse-fine
 // fluxes to cf for flux matching.  One tile of the stencil list per block.
 // In flux form (each face's two tangent fluxes, then the divergence) a cell
 // took 40 FP64 instructions and the kernel was bound by the FP64 pipe; the
 // rows move 9% more bytes.  Its four plain products run on the integer pipe.
-// At 256^3: 1.30 -> 0.73 ms (six blocks per SM; with five 0.78): 0.90 of the
-// FP64 issue rate, the bound left, and 0.63 of HBM.  The row's order costs
-// 0.04 ms against own entries first, whose rounding error is a fifth larger
-// (2.5e-16 in the 2-norm against 2.1e-16 here, 2.2e-16 in flux form).
+// At 256^3: 1.30 -> 0.73 ms (six blocks per SM; with five 0.78): 0.93 of the
+// FP64 issue rate, the bound left, and 0.63 of HBM.  Rounding: a row's order costs
+// 0.04 ms against own entries first, whose error with the coefficients given is a
+// fifth larger (2.5e-16 against 2.1e-16 in the 2-norm).  The product's distance
+// from a 64-bit evaluation of the whole chain is 2.5-2.6e-16 at 256^3, 2.3e-16 in
+// flux form: the own entries are sums, rounded before they meet the vector.
 // MINB < 6 (few tiles, launch_jv_frozen): the loads of several faces in flight,
 // and every cell by the boundary's path, since the cells of small patches mostly
 // take it and a warp holding both takes them in turn.
