@@ -192,3 +192,25 @@ def test_boxes_both_forms(nrd, n0, levels):
         exp = R.regrid_boxes(h, tags, tag_bits=2, buffer=buf, efficiency=eff, min_side=mn,
                              max_side=mx, max_levels=ml)
         assert as_lists(got) == as_lists(exp)
+
+
+def test_tags_of_a_captured_call(nrd):
+    """nrd_tag in a CUDA graph, replayed on new states: the clustering takes the
+    replay's tags."""
+    h = W.uniform(24)
+    u = dev(W.front_state(h, seed=4, noise=0.0, front=0.4, width=0.1))
+    late = dev(W.front_state(h, seed=4, noise=0.0, front=0.6, width=0.1))
+    ctx = ctx_for(nrd, h)
+    boxes = lambda t: as_lists(ctx.regrid_boxes(t, 4, 1, 0.7, 4, 16, 2))  # noqa: E731
+    exp = [boxes(ctx.tag(x, thr_r=0.1)) for x in (u, late)]
+    assert exp[0] != exp[1]
+    v, s, g = u.clone(), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s):
+        tags = ctx.tag(v, thr_r=0.1)
+    with torch.cuda.stream(s):
+        for x, e in zip((u, late), exp):
+            torch.cuda._sleep(100_000_000)
+            v.copy_(x)
+            g.replay()
+            assert boxes(tags) == e
