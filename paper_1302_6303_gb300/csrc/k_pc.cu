@@ -740,11 +740,16 @@ __device__ __forceinline__ void k_lsmooth_tile(const VItem& it, VLev<P> V, int c
   }
 }
 
+// (FP64: registers for five blocks per SM; left to itself the compiler takes 40
+// for the later passes and keeps fewer loads in flight: a pass on the patches of an
+// 8^3 base 11.7 against 10.9 us, on a 64^3 base with a fine band 21.3 against 20.9.
+// With four a V-cycle on the latter takes 448 us against 443.  FP32: its own choice,
+// 32 to 40; on 250 patches, 5.7M cells, a bound of four or five is slower, 81 and 70
+// against 65 us.)
 template <class P, bool ZERO, bool ADD>
-__global__ void __launch_bounds__(VTHREADS) k_lsmooth(int ntl, VLev<P> V, int t0, int colour,
-                                                      P* __restrict__ e,
-                                                      const P* __restrict__ f,
-                                                      P* __restrict__ u) {
+__global__ void __launch_bounds__(VTHREADS, sizeof(P) > 4 ? 5 : 0)
+k_lsmooth(int ntl, VLev<P> V, int t0, int colour, P* __restrict__ e, const P* __restrict__ f,
+          P* __restrict__ u) {
   tile_loop<(sizeof(P) > 4)>(ntl, V.vt + t0, [&](const VItem& it) {
     k_lsmooth_tile<P, ZERO, ADD>(it, V, colour, e, f, u);
   });
